@@ -16,10 +16,11 @@
 // of that (2H)-square system gives every H' at once (Sec. 1).  Everything is
 // normalised by W and sqrt(W chi2_poly), so Delta chi^2' lies in [0, 1].
 //
-// One warp per trial frequency in double: lane l holds harmonic column l + 1.
-// The gridded pass flags bins whose estimated error is too large; those, and
-// the records, are recomputed from exact double sums over the samples (the Q
-// and P sums of the double fix-up tier plus the trend sums T).
+// The gridded pass solves one trial frequency per thread in double and flags
+// bins whose estimated error is too large; those, and the records, are
+// recomputed from exact double sums over the samples (the Q and P sums of the
+// double fix-up tier plus the trend sums T), one warp per bin: lane l holds
+// harmonic column l + 1.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -41,20 +42,19 @@ struct JointParams {
     double chi0;     // chi2_poly
     double LG[16];   // normalised polynomial Gram factor, lower triangle, row-major 4 x 4
     double yP[4];    // L_G^-1 beta_P (normalised)
+    double iLG[4];   // 1 / L_G[p][p]
 };
 
 // Harmonic-column solve of the projected system for one bin.  S holds the
 // normalised Q (qr/qi, k = 0..2H) and P (pr/pi, k = 1..H) sums, T the
 // normalised trend sums T_{p,h} at [(p - 1) H + h - 1] (re, im).  Every lane
-// returns out[H' - 1] = Delta chi^2'_{H'} and the smallest relative pivot.
-// With COEF, *anorm2 = max over H' <= H of the harmonic coefficient norm
-// |A_H'|^2 (float, for the error estimate); with coef != nullptr, coef[0..2Hc)
+// returns out[H' - 1] = Delta chi^2'_{H'}; with coef != nullptr, coef[0..2Hc)
 // gets the Hc-harmonic coefficients and poly[0..D] the polynomial ones
 // (normalised units).
-template <int H, int D, bool COEF>
-FC2_D double warp_joint_solve(const Sys<double, H>& S, const double* Tre, const double* Tim,
-                              const JointParams& jp, double* out, double* anorm2,
-                              double* coef = nullptr, int Hc = 0, double* poly = nullptr) {
+template <int H, int D>
+FC2_D void warp_joint_solve(const Sys<double, H>& S, const double* Tre, const double* Tim,
+                            const JointParams& jp, double* out, double* coef = nullptr,
+                            int Hc = 0, double* poly = nullptr) {
     constexpr int m = 2 * H;
     static_assert(m <= 32, "one column per lane");
     constexpr unsigned FULL = 0xffffffffu;
@@ -99,7 +99,6 @@ FC2_D double warp_joint_solve(const Sys<double, H>& S, const double* Tre, const 
     // right-looking Cholesky, lane l holding row l
     double Lr[m], z[m], dinv[m];
     double acc = 0.0;
-    float dmin = 1.0f;
 #pragma unroll
     for (int k = 0; k < m; ++k) {
         const double dk = __shfl_sync(FULL, a[k], k);
@@ -118,31 +117,8 @@ FC2_D double warp_joint_solve(const Sys<double, H>& S, const double* Tre, const 
             if (j <= l) a[j] = fma(-Llk, Ljk, a[j]);
         }
         b = fma(-Llk, zk, b);
-        const float rc = allk > 0.0 ? fmaxf((float)dk / (float)allk, 0.0f) : 0.0f;
-        dmin = fminf(dmin, rc);
         acc = fma(zk, zk, acc);
         if ((k & 1) == 1) out[k >> 1] = acc;
-    }
-    if constexpr (COEF) {
-        float amax = 0.0f;
-#pragma unroll
-        for (int hp = 1; hp <= H; ++hp) {
-            const int mp = 2 * hp;
-            float mine = 0.0f, nrm = 0.0f;
-#pragma unroll
-            for (int k = m - 1; k >= 0; --k) {
-                if (k < mp) {
-                    float t = (l > k && l < mp) ? (float)Lr[k] * mine : 0.0f;
-#pragma unroll
-                    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(FULL, t, o);
-                    const float A = ((float)z[k] - t) * (float)dinv[k];
-                    if (l == k) mine = A;
-                    nrm = fmaf(A, A, nrm);
-                }
-            }
-            amax = fmaxf(amax, nrm);
-        }
-        *anorm2 = (double)amax;
     }
     if (coef) {
         const int mp = 2 * Hc;
@@ -177,14 +153,31 @@ FC2_D double warp_joint_solve(const Sys<double, H>& S, const double* Tre, const 
             poly[p] = v / jp.LG[p * 4 + p];
         }
     }
-    return (double)dmin;
 }
 
 // ---------------------------------------------------------- gridded pass
-// Warp per bin.  Spectra rows: Q_1..Q_2H, P_1..P_H, then T_{p,1..H} for
+// One thread per bin.  Spectra rows: Q_1..Q_2H, P_1..P_H, then T_{p,1..H} for
 // p = 1..D (all deconvolved by dec[j]).  Bins whose error estimate is too
 // large, or whose smallest relative pivot is below what these sums resolve,
 // go to the exact list.
+//
+// Bound by the double pipe: one double instruction of a warp holds its
+// sub-partition for 64 clocks however many lanes are active, so the solve is
+// laid out to fill all 32 lanes (a warp per bin, with 2H lanes active and every
+// lane repeating the loads and scalings, spent 16 times the instructions) and
+// nothing that double arithmetic need not do stays on it: the spectra are
+// widened by integer operations, the factor 1/2 of the alpha entries is folded
+// into their scale, the divisions by L_G's diagonal are products with its
+// reciprocals, and the coefficient norm, which only feeds the error estimate,
+// is formed in float.  About 520 double operations per bin at H = 4, D = 2.
+// Spilled rows cost little beside them.  N = 2^18, H = 4, D = 2, float
+// spectra: 6036 -> 313 us (double pipe alone: about 220 us).
+FC2_D double widen(float v) { return f2d_exact(v); }
+FC2_D double widen(double v) { return v; }
+// double -> float for the error estimate, on the integer pipes (truncating;
+// magnitudes outside the float range give 0 or infinity).
+FC2_D float narrow_est(double v) { return copysignf(d2f_trunc(fabs(v)), (float)(__double2hiint(v) >> 31 | 1)); }
+
 template <typename TS, int H, int D>
 __global__ void __launch_bounds__(128) k_assemble_joint(const cpx<TS>* __restrict__ spec,
                                                         const TS* __restrict__ dec,
@@ -193,42 +186,116 @@ __global__ void __launch_bounds__(128) k_assemble_joint(const cpx<TS>* __restric
                                                         int32_t* __restrict__ list,
                                                         int32_t* __restrict__ list_count,
                                                         int64_t cap) {
-    const int64_t wpb = blockDim.x >> 5;
-    for (int64_t j = (int64_t)blockIdx.x * wpb + (threadIdx.x >> 5); j < jp.N;
-         j += (int64_t)gridDim.x * wpb) {
-        const double d = (double)dec[j];
-        const double dq = d * jp.sq, dp = d * jp.jsp;
-        Sys<double, H> S;
-        S.qr[0] = 1.0; S.qi[0] = 0.0; S.pr[0] = 0.0; S.pi[0] = 0.0;
+    constexpr int m = 2 * H;
+    const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (j >= jp.N) return;
+    const double d = widen(dec[j]);
+    const double dq = d * jp.sq, dqh = 0.5 * dq, dp = d * jp.jsp;
+    double qr[2 * H + 1], qi[2 * H + 1];  // halves of the normalised Q sums
+    qr[0] = 0.5;
+    qi[0] = 0.0;
 #pragma unroll
-        for (int k = 1; k <= 2 * H; ++k) {
-            const cpx<TS> v = spec[(int64_t)(k - 1) * jp.N + j];
-            S.qr[k] = (double)v.x * dq;
-            S.qi[k] = (double)v.y * dq;
+    for (int k = 1; k <= 2 * H; ++k) {
+        const cpx<TS> v = spec[(int64_t)(k - 1) * jp.N + j];
+        qr[k] = widen(v.x) * dqh;
+        qi[k] = widen(v.y) * dqh;
+    }
+    // columns c = 1..2H of the unprojected system (odd: sine, even: cosine):
+    // cross terms with the polynomial, projected (Y = L_G^-1 C), and the rhs
+    double Y[m][D + 1], b[m];
+#pragma unroll
+    for (int h = 1; h <= H; ++h) {
+        const cpx<TS> pv = spec[(int64_t)(2 * H + h - 1) * jp.N + j];
+        b[2 * h - 2] = widen(pv.y) * dp;
+        b[2 * h - 1] = widen(pv.x) * dp;
+        double cs[D + 1], cc[D + 1];
+        cs[0] = qi[h] + qi[h];
+        cc[0] = qr[h] + qr[h];
+#pragma unroll
+        for (int p = 1; p <= D; ++p) {
+            const cpx<TS> v = spec[(int64_t)(3 * H + (p - 1) * H + h - 1) * jp.N + j];
+            cs[p] = widen(v.y) * dq;
+            cc[p] = widen(v.x) * dq;
         }
 #pragma unroll
-        for (int k = 1; k <= H; ++k) {
-            const cpx<TS> v = spec[(int64_t)(2 * H + k - 1) * jp.N + j];
-            S.pr[k] = (double)v.x * dp;
-            S.pi[k] = (double)v.y * dp;
-        }
-        double Tre[D * H], Tim[D * H];
+        for (int p = 0; p <= D; ++p) {
+            double vs = cs[p], vc = cc[p];
 #pragma unroll
-        for (int q = 0; q < D * H; ++q) {
-            const cpx<TS> v = spec[(int64_t)(3 * H + q) * jp.N + j];
-            Tre[q] = (double)v.x * dq;
-            Tim[q] = (double)v.y * dq;
-        }
-        double out[H], an2 = 0.0;
-        const double dmin = warp_joint_solve<H, D, true>(S, Tre, Tim, jp, out, &an2);
-        if ((threadIdx.x & 31) == 0) {
-            if (!(est_err<double>(an2, 2 * H + 1 + D, jp.eps) <= jp.err_fix) || dmin < dmin_exact) {
-                const int32_t pos = atomicAdd(list_count, 1);
-                if (pos < cap) list[pos] = (int32_t)j;
+            for (int q = 0; q < p; ++q) {
+                vs = fma(-jp.LG[p * 4 + q], Y[2 * h - 2][q], vs);
+                vc = fma(-jp.LG[p * 4 + q], Y[2 * h - 1][q], vc);
             }
-#pragma unroll
-            for (int hh = 0; hh < H; ++hh) dchi2[(int64_t)hh * jp.N + j] = out[hh] * jp.chi0;
+            Y[2 * h - 2][p] = vs * jp.iLG[p];
+            Y[2 * h - 1][p] = vc * jp.iLG[p];
         }
+    }
+    // nested Cholesky of the projected harmonic block, row by row
+    double L[m][m], dinv[m], z[m];
+    float Lf[m][m];
+    double acc = 0.0;
+    float dmin = 1.0f;
+#pragma unroll
+    for (int l = 0; l < m; ++l) {
+        const int hl = (l + 2) >> 1;
+        const bool sl = ((l + 1) & 1) != 0;
+#pragma unroll
+        for (int k = 0; k <= l; ++k) {
+            const int hk = (k + 2) >> 1, s = hl + hk, dd = hl - hk;  // hl >= hk
+            const bool sk = ((k + 1) & 1) != 0;
+            double v;
+            if (sl && sk) v = qr[dd] - qr[s];
+            else if (!sl && !sk) v = qr[dd] + qr[s];
+            else if (sl) v = dd > 0 ? qi[s] + qi[dd] : qi[s];  // sin(hl) cos(hk)
+            else v = dd > 0 ? qi[s] - qi[dd] : qi[s];          // cos(hl) sin(hk)
+#pragma unroll
+            for (int p = 0; p <= D; ++p) v = fma(-Y[l][p], Y[k][p], v);
+            const double projected = v;
+#pragma unroll
+            for (int p = 0; p < k; ++p) v = fma(-L[l][p], L[k][p], v);
+            if (k < l) {
+                L[l][k] = v * dinv[k];
+                Lf[l][k] = narrow_est(L[l][k]);
+            } else {
+                const bool keep = projected > 0.0 && v > jp.tau * projected;
+                dinv[l] = keep ? rsqrt(v) : 0.0;
+                const float rc = projected > 0.0
+                                     ? fmaxf(narrow_est(v) / d2f_trunc(projected), 0.0f) : 0.0f;
+                dmin = fminf(dmin, rc);
+            }
+        }
+        double v = b[l];
+#pragma unroll
+        for (int p = 0; p <= D; ++p) v = fma(-Y[l][p], jp.yP[p], v);
+#pragma unroll
+        for (int k = 0; k < l; ++k) v = fma(-L[l][k], z[k], v);
+        z[l] = v * dinv[l];
+        acc = fma(z[l], z[l], acc);
+        if ((l & 1) == 1) dchi2[(int64_t)(l >> 1) * jp.N + j] = acc * jp.chi0;
+    }
+    // largest coefficient norm over the nested models, by back-substitution
+    float zf[m], df[m], amax = 0.0f;
+#pragma unroll
+    for (int l = 0; l < m; ++l) { zf[l] = narrow_est(z[l]); df[l] = narrow_est(dinv[l]); }
+#pragma unroll
+    for (int mp = 2; mp <= m; mp += 2) {
+        float A[m], nrm = 0.0f;
+#pragma unroll
+        for (int k = m - 1; k >= 0; --k) {
+            if (k < mp) {
+                float t = zf[k];
+#pragma unroll
+                for (int l = k + 1; l < m; ++l)
+                    if (l < mp) t = fmaf(-Lf[l][k], A[l], t);
+                A[k] = t * df[k];
+                nrm = fmaf(A[k], A[k], nrm);
+            }
+        }
+        amax = fmaxf(amax, nrm);
+    }
+    if (!(est_err<double>((double)amax, 2 * H + 1 + D, jp.eps) <= jp.err_fix) ||
+        (double)dmin < dmin_exact) {
+        const int32_t pos = atomicAdd(list_count, 1);
+        if (pos < cap) list[pos] = (int32_t)j;
     }
 }
 
@@ -351,8 +418,8 @@ __global__ void __launch_bounds__(128) k_exact_joint_dchi2(
     Sys<double, H> S;
     double Tre[D * H], Tim[D * H];
     joint_exact_sys<H, D>(part, part_t, b, nch, scal, sh[w], sht[w], S, Tre, Tim);
-    double out[H], an2 = 0.0;
-    warp_joint_solve<H, D, false>(S, Tre, Tim, jp, out, &an2);
+    double out[H];
+    warp_joint_solve<H, D>(S, Tre, Tim, jp, out);
     if ((threadIdx.x & 31) != 0) return;
     const int64_t j = list[base + b];
 #pragma unroll
@@ -385,8 +452,8 @@ __global__ void __launch_bounds__(128) k_exact_joint_coeffs(
     Sys<double, H> S;
     double Tre[D * H], Tim[D * H];
     joint_exact_sys<H, D>(part, part_t, r, nch, scal, sh[w], sht[w], S, Tre, Tim);
-    double o[H], an2 = 0.0, coef[2 * H], poly[D + 1];
-    warp_joint_solve<H, D, false>(S, Tre, Tim, jp, o, &an2, coef, Hp, poly);
+    double o[H], coef[2 * H], poly[D + 1];
+    warp_joint_solve<H, D>(S, Tre, Tim, jp, o, coef, Hp, poly);
     if ((threadIdx.x & 31) != 0) return;
     const double W = scal[SC_W];
     const double unit = (W > 0.0) ? sqrt(jp.chi0 / W) : 0.0;
@@ -418,7 +485,10 @@ static JointParams joint_params(const fc2_plan_s* p) {
     jp.chi0 = p->jt_chi0;
     jp.jsp = (p->jt_chi0 > 0.0) ? 1.0 / sqrt(p->scal[SC_W] * p->jt_chi0) : 0.0;
     for (int i = 0; i < 16; ++i) jp.LG[i] = p->jt_LG[i];
-    for (int i = 0; i < 4; ++i) jp.yP[i] = p->jt_yP[i];
+    for (int i = 0; i < 4; ++i) {
+        jp.yP[i] = p->jt_yP[i];
+        jp.iLG[i] = p->jt_LG[i * 4 + i] > 0.0 ? 1.0 / p->jt_LG[i * 4 + i] : 0.0;
+    }
     return jp;
 }
 
@@ -430,7 +500,7 @@ static cudaError_t assemble_joint_impl(fc2_plan_s* p, cudaStream_t s) {
     int32_t* cnt = p->d_flag_count + 3;
     const cpx<TS>* spec = (const cpx<TS>*)p->d_spec;
     const TS* dec = (const TS*)p->d_dec;
-    const unsigned blocks = (unsigned)std::min<int64_t>((p->N + 3) / 4, 152 * 64);
+    const unsigned blocks = (unsigned)((p->N + 127) / 128);
     const double dmin_exact = p->fp64 ? 1e-11 : 1e-7;
 #define FC2_JA(HH, DD)                                                                        \
     if (p->H == HH && p->D == DD) {                                                           \
