@@ -302,6 +302,7 @@ struct AdjTab {
     const int32_t* perm;     // sorted position -> caller position (global), or null
     const int64_t* ent;      // [E] (curve << 32 | j)
     const double* gout;      // [E] upstream gradients or null (= 1)
+    const double2* phasors;  // [512] the double phasor tables (launch_init_dftab's second part)
     int K;                   // entries per curve (output layout of d_dx / d_dsigma)
     double tol;              // Newton stopping step
     int max_iter;

@@ -2291,7 +2291,7 @@ fc2_status batched_backward(int64_t C, const int64_t* offsets, const double* t, 
     int64_t* off = nullptr; int* Hd = nullptr; double *fm = nullptr, *dfd = nullptr, *scal = nullptr;
     int32_t *perm = nullptr, *status = nullptr; double *tau = nullptr, *wq = nullptr, *wp = nullptr;
     uint64_t *A = nullptr, *B = nullptr; float *w32 = nullptr, *p32 = nullptr;
-    int64_t* ent = nullptr; double* g = nullptr;
+    int64_t* ent = nullptr; double* g = nullptr; void* dftab = nullptr;
     double *of = nullptr, *od = nullptr, *og = nullptr, *oxx = nullptr, *oss = nullptr;
     alloc((void**)&off, (C + 1) * 8); alloc((void**)&Hd, C * 4); alloc((void**)&fm, C * 8);
     alloc((void**)&dfd, C * 8); alloc((void**)&scal, C * SC_COUNT * 8); alloc((void**)&status, 16);
@@ -2299,7 +2299,7 @@ fc2_status batched_backward(int64_t C, const int64_t* offsets, const double* t, 
     alloc((void**)&wp, ntot * 8); alloc((void**)&A, ntot * 8); alloc((void**)&B, ntot * 8);
     // float weights: high parts at [i], low parts at [ntot + i]
     alloc((void**)&w32, 2 * ntot * 4); alloc((void**)&p32, 2 * ntot * 4);
-    alloc((void**)&ent, E * 8);
+    alloc((void**)&ent, E * 8); alloc(&dftab, 2 * 512 * 16);
     alloc((void**)&of, E * 8); alloc((void**)&od, E * 8); alloc((void**)&og, E * 8);
     if (grad_out) alloc((void**)&g, E * 8);
     const bool dx_dev = is_dev(d_dx), ds_dev = is_dev(d_dsig);
@@ -2321,12 +2321,14 @@ fc2_status batched_backward(int64_t C, const int64_t* offsets, const double* t, 
         cudaMemcpyAsync(ent, entv.data(), E * 8, cudaMemcpyHostToDevice, s);
         if (grad_out) cudaMemcpyAsync(g, grad_out, E * 8, cudaMemcpyDefault, s);
         cudaMemsetAsync(status, 0, 16, s);
+        const cudaError_t et = launch_init_dftab(dftab, false, s);
         launch_moments(dt, dx, ds, off, C, 0, scal, status, s);
         std::vector<double> hs((size_t)C * SC_COUNT);
         int32_t hst = 0;
         cudaMemcpyAsync(hs.data(), scal, hs.size() * 8, cudaMemcpyDeviceToHost, s);
         cudaMemcpyAsync(&hst, status, 4, cudaMemcpyDeviceToHost, s);
         e = cudaStreamSynchronize(s);
+        if (e == cudaSuccess) e = et;
         if (e == cudaSuccess && hst) st = (fc2_status)hst;
         if (e == cudaSuccess && st == FC2_OK) {
             k_iota_plus<<<(unsigned)((ntot + 255) / 256), 256, 0, s>>>(perm, ntot, 0);
@@ -2342,7 +2344,8 @@ fc2_status batched_backward(int64_t C, const int64_t* offsets, const double* t, 
             k_bgather<<<(unsigned)((ntot + 255) / 256), 256, 0, s>>>(dt, dx, ds, perm, ntot, off, (int)C,
                                                                     scal, fm, dfd, tau, wq, wp, A, B,
                                                                     w32, p32);
-            AdjTab tb{off, Hd, fm, dfd, scal, tau, wq, wp, perm, ent, g, K, 1e-10, 40};
+            AdjTab tb{off, Hd, fm, dfd, scal, tau, wq, wp, perm, ent, g,
+                      reinterpret_cast<const double2*>(dftab) + 512, K, 1e-10, 40};
             AdjOut out{of, od, og, d_dx ? (dx_dev ? d_dx : oxx) : nullptr,
                        d_dsig ? (ds_dev ? d_dsig : oss) : nullptr};
             if (e == cudaSuccess) e = launch_backward_tab(tb, E, out, s);
