@@ -312,6 +312,7 @@ template <int TIER>
 struct BxTables {
     dfc t2[(TIER == 2 || TIER == 4) ? 512 : 1];
     double2 t3[TIER == 3 ? 512 : 1];
+    FxStage<1> stage[TIER == 4 ? BX_W : 1];  // tier 4: each warp's staged samples
     FC2_D void load(const dfc* __restrict__ dftab) {
         if constexpr (TIER == 2 || TIER == 4)
             for (int i = threadIdx.x; i < 512; i += blockDim.x) t2[i] = dftab[i];
@@ -330,7 +331,7 @@ template <int HM, int TIER>
 FC2_D void bx_sums(const uint64_t* __restrict__ Aph, const uint64_t* __restrict__ Bph,
                    const float* __restrict__ wq32, const float* __restrict__ wp32,
                    const double* __restrict__ wq, const double* __restrict__ wp,
-                   const BxTables<TIER>& tb, int64_t ntot, uint64_t ju, int H, int64_t i0,
+                   BxTables<TIER>& tb, int64_t ntot, uint64_t ju, int H, int64_t i0,
                    int64_t i1, int lane, double* tot) {
     constexpr int NV = 6 * HM;
     if constexpr (TIER == 1) {
@@ -388,10 +389,6 @@ FC2_D void bx_sums(const uint64_t* __restrict__ Aph, const uint64_t* __restrict_
             tot[v] = (double)x.x + (double)x.y;
         }
     } else if constexpr (TIER == 4) {
-        // lph lanes per harmonic multiple k = 1..2H (lane = (k - 1) lph + r),
-        // each over the samples i0 + r, + lph, ..; sums exact in fixed point
-        const int lph = 32 / (2 * H);
-        const int g = lane / lph, r = lane - g * lph;
         float mq = 0.f, mp = 0.f;  // the item's largest weights set the scales
         for (int64_t i = i0 + lane; i < i1; i += 32) {
             mq = fmaxf(mq, fabsf(wq32[i]));
@@ -402,31 +399,22 @@ FC2_D void bx_sums(const uint64_t* __restrict__ Aph, const uint64_t* __restrict_
         // a harmonic's terms over the item (|w e^{..}| <= |w| (1 + 2^-23))
         const int eq = fx_exponent(mq * 1.0000002f, i1 - i0 + 1);
         const int ep = fx_exponent(mp * 1.0000002f, i1 - i0 + 1);
-        long long acc[4] = {0, 0, 0, 0};
-        if (g < 2 * H)
-            fx_lane_sums<false>(Aph, Bph, wq32, wp32, ntot, ju, (uint64_t)(g + 1), i0, i1, r, lph,
-                                g < H, tb.t2, tb.t2 + 256, exp2f((float)eq), exp2f((float)ep), acc);
-        // group sums, exact: the group's first lane adds its lanes' values in order
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            long long s = acc[q];
-            for (int o = 1; o < lph; ++o) {
-                const long long y = __shfl_sync(0xffffffffu, acc[q], (lane + o) & 31);
-                if (r == 0) s += y;
-            }
-            acc[q] = s;
-        }
+        const int lph = 32 / (2 * H);
+        FxSums fx = fx_group_sums<false, 1>(tb.stage[threadIdx.x >> 5], Aph, Bph, wq32, wp32, ntot,
+                                            ju, H, i0, i1, tb.t2, tb.t2 + 256, exp2f((float)eq),
+                                            exp2f((float)ep));
+        fx_group_sum(fx, H);
         const double uq = ldexp(1.0, -eq), up = ldexp(1.0, -ep);
 #pragma unroll
         for (int k = 0; k < 2 * HM; ++k) {
-            const int src = (k < 2 * H) ? k * lph : 0;
-            const double v0 = (double)__shfl_sync(0xffffffffu, acc[0], src) * uq;
-            const double v1 = (double)__shfl_sync(0xffffffffu, acc[1], src) * uq;
-            const double v2 = (double)__shfl_sync(0xffffffffu, acc[2], src) * up;
-            const double v3 = (double)__shfl_sync(0xffffffffu, acc[3], src) * up;
+            const int src = (k < 2 * H) ? (k < H ? k : k - H) * 2 * lph : 0;
+            const double v0 = (double)__shfl_sync(0xffffffffu, k < H ? fx.q[0][0] : fx.q[1][0], src) * uq;
+            const double v1 = (double)__shfl_sync(0xffffffffu, k < H ? fx.q[0][1] : fx.q[1][1], src) * uq;
             tot[2 * k] = (k < 2 * H) ? v0 : 0.0;
             tot[2 * k + 1] = (k < 2 * H) ? v1 : 0.0;
             if (k < HM) {
+                const double v2 = (double)__shfl_sync(0xffffffffu, fx.p[0], src) * up;
+                const double v3 = (double)__shfl_sync(0xffffffffu, fx.p[1], src) * up;
                 tot[4 * HM + 2 * k] = (k < H) ? v2 : 0.0;
                 tot[4 * HM + 2 * k + 1] = (k < H) ? v3 : 0.0;
             }
@@ -531,7 +519,7 @@ __global__ void __launch_bounds__(BX_SPLIT_NT) k_bx_split(CurveTab ct,
 // One warp per work item: the item's share of its entry's samples, summed
 // into row w of part (6 BHM doubles per row).
 template <int HM, int TIER>
-__global__ void __launch_bounds__(BX_NT) k_bx_part(
+__global__ void __launch_bounds__(BX_NT, TIER == 4 ? 2 : 1) k_bx_part(
     const uint64_t* __restrict__ Aph, const uint64_t* __restrict__ Bph,
     const float* __restrict__ wq32, const float* __restrict__ wp32,
     const double* __restrict__ wq, const double* __restrict__ wp, const dfc* __restrict__ dftab,

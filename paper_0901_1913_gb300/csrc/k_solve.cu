@@ -281,7 +281,7 @@ __global__ void k_phase_fx(const double* __restrict__ tau, const double* __restr
 // Tables e^{2 pi i a / 256} (entries 0..255) and e^{2 pi i b / 65536}
 // (entries 256..511): double-float for df_phasor (tier 2), then the same in
 // double (tier 3); then e^{2 pi i m / 65536}, m < 65536, double-float, for
-// df_phasor16 (the last tier) at DFTAB_T16.
+// the last tier (df2_table16) at DFTAB_T16.
 __global__ void k_init_dftab(dfc* __restrict__ tab, int with16) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= (with16 ? 512 + 65536 : 512)) return;
@@ -313,7 +313,7 @@ FC2_D float2 warp_sum_pair(float hi, float lo) {
 }
 
 template <int HM, int TIER>
-__global__ void __launch_bounds__(EX_NT) k_exact_partial(
+__global__ void __launch_bounds__(EX_NT, TIER == 4 ? EX_MINB : 1) k_exact_partial(
     const uint64_t* __restrict__ Aph, const uint64_t* __restrict__ Bph,
     const float* __restrict__ wq32, const float* __restrict__ wp32,
     const double* __restrict__ wq, const double* __restrict__ wp, const dfc* __restrict__ dftab,
@@ -327,6 +327,7 @@ __global__ void __launch_bounds__(EX_NT) k_exact_partial(
     __shared__ dfc stab[TIER == 2 ? 512 : 1];
     __shared__ double2 stab64[TIER == 3 ? 512 : 1];
     __shared__ float smax[2][EX_NT / 32];
+    __shared__ FxStage<TIER == 4 ? EX_NT / 32 : 0> fxst;
     int64_t cnt = count_dev ? (int64_t)(*count_dev) - base : count;
     if (cnt > cap) cnt = cap;
     if (cnt <= 0) return;
@@ -406,9 +407,7 @@ __global__ void __launch_bounds__(EX_NT) k_exact_partial(
                 if (lane == 0) redf[wpi][v] = x;
             }
         } else if constexpr (TIER == 4) {
-            // lph lanes per harmonic multiple k (lane = (k - 1) lph + r); warp w
-            // takes samples i0 + r + lph (w + 8 q); sums exact in fixed point at
-            // scales set by the item's largest weights
+            // sums exact in fixed point at scales set by the item's largest weights
             float mq = 0.f, mp = 0.f;
             for (int64_t i = i0 + threadIdx.x; i < i1; i += EX_NT) {
                 mq = fmaxf(mq, fabsf(wq32[i]));
@@ -426,29 +425,18 @@ __global__ void __launch_bounds__(EX_NT) k_exact_partial(
             const int eq = fx_exponent(mq * 1.0000002f, i1 - i0 + 1);
             const int ep = fx_exponent(mp * 1.0000002f, i1 - i0 + 1);
             const int lph = 32 / (2 * H);
-            const int g = lane / lph, r = lane - g * lph;
-            long long acc[4] = {0, 0, 0, 0};
-            if (g < 2 * H)
-                fx_lane_sums<true>(Aph, Bph, wq32, wp32, n, ju, (uint64_t)(g + 1), i0, i1,
-                                   r + (int64_t)lph * wpi, (int64_t)lph * (EX_NT / 32), g < H,
-                                   dftab + DFTAB_T16, nullptr, exp2f((float)eq),
-                                   exp2f((float)ep), acc);
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                long long sacc = acc[q];
-                for (int o = 1; o < lph; ++o) {
-                    const long long y = __shfl_sync(0xffffffffu, acc[q], (lane + o) & 31);
-                    if (r == 0) sacc += y;
-                }
-                acc[q] = sacc;
-            }
-            if (r == 0 && g < 2 * H) {
+            FxSums fx = fx_group_sums<true, EX_NT / 32>(fxst, Aph, Bph, wq32, wp32, n, ju, H, i0,
+                                                        i1, dftab + DFTAB_T16, nullptr,
+                                                        exp2f((float)eq), exp2f((float)ep));
+            fx_group_sum(fx, H);
+            const int g = lane / (2 * lph);
+            if (lane == 2 * lph * g && g < H) {
                 const double uq = ldexp(1.0, -eq), up = ldexp(1.0, -ep);
-                red[wpi][2 * g] = (double)acc[0] * uq;
-                red[wpi][2 * g + 1] = (double)acc[1] * uq;
-                if (g < H) {
-                    red[wpi][4 * HM + 2 * g] = (double)acc[2] * up;
-                    red[wpi][4 * HM + 2 * g + 1] = (double)acc[3] * up;
+#pragma unroll
+                for (int v = 0; v < 2; ++v) {
+                    red[wpi][2 * g + v] = (double)fx.q[0][v] * uq;
+                    red[wpi][2 * (g + H) + v] = (double)fx.q[1][v] * uq;
+                    red[wpi][4 * HM + 2 * g + v] = (double)fx.p[v] * up;
                 }
             }
             // values of multiples beyond 2H (and P beyond H) are never read
@@ -1022,12 +1010,14 @@ cudaError_t launch_init_dftab(void* tab, bool with16, cudaStream_t s) {
 }
 
 // The double-float phasor of each phase (diagnostics: its accuracy test), from
-// the two 256-entry tables (df_phasor) or the 65536-entry one (df_phasor16).
+// the two 256-entry tables or the 65536-entry one, as the last tier forms it.
 __global__ void k_debug_phasor(const uint64_t* __restrict__ u, int64_t n,
                                const dfc* __restrict__ tab, int table16, float* __restrict__ out) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    const dfc z = table16 ? df_phasor16(u[i], tab + DFTAB_T16) : df_phasor(u[i], tab, tab + 256);
+    const dfc2 z2 = table16 ? df2_rotate<true>(u[i], u[i], df2_table16(u[i], u[i], tab + DFTAB_T16))
+                            : df2_rotate<false>(u[i], u[i], df2_table(u[i], u[i], tab, tab + 256));
+    const dfc z{{z2.re.h.x, z2.re.l.x}, {z2.im.h.x, z2.im.l.x}};
     out[4 * i] = z.re.h;
     out[4 * i + 1] = z.re.l;
     out[4 * i + 2] = z.im.h;
