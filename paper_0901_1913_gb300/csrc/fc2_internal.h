@@ -145,6 +145,7 @@ struct fc2_plan_s {
     int64_t twst_off[16] = {0};
     int64_t tw64_off[16] = {0};
     int fft_family = fc2::FFT_R64;  // kernel family of the float passes (fc2::FftFamily)
+    bool fused_fft = false;    // double passes by k_fft_pass_d (batches, whose results are float)
     int fft_group = 0;         // grids taken through all passes together (0 = all)
     int spread_tile = 0;       // cells per spreading tile (0 = default for M)
     double* d_dchi2 = nullptr; // [H][N]
@@ -236,6 +237,7 @@ cudaError_t launch_detrend(const double* t, const double* x, const double* sigma
                            cudaStream_t s);
 
 // k_fft.cu
+void twiddle_split(int logM, bool fused, int* sh, int64_t* nlo, int64_t* nhi);  // d_twlo, d_twhi entries
 cudaError_t init_twiddles(fc2_plan_s* p, cudaStream_t s);
 cudaError_t init_deconv(fc2_plan_s* p, cudaStream_t s);
 void plan_fft_passes(fc2_plan_s* p);

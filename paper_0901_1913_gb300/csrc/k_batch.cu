@@ -1844,9 +1844,12 @@ fc2_status batched_execute(int64_t C, const int64_t* offsets, const double* t, c
             plan_fft_passes(&p);
             p.fft_family = fft_family_of(opt.fft_kernel);
             release(p.d_twlo, s); release(p.d_twhi, s); release(p.d_twst, s); release(p.d_dec, s);
-            const int sh = (p.logM + 1) / 2;
-            cudaError_t ea = pool_alloc((void**)&p.d_twlo, (size_t)(1ll << sh) * csz, s);
-            if (ea == cudaSuccess) ea = pool_alloc((void**)&p.d_twhi, (size_t)(M >> sh) * csz, s);
+            int sh;
+            int64_t nlo, nhi;
+            p.fused_fft = fp64;
+            twiddle_split(p.logM, p.fused_fft, &sh, &nlo, &nhi);
+            cudaError_t ea = pool_alloc((void**)&p.d_twlo, (size_t)nlo * csz, s);
+            if (ea == cudaSuccess) ea = pool_alloc((void**)&p.d_twhi, (size_t)nhi * csz, s);
             if (ea == cudaSuccess) ea = pool_alloc((void**)&p.d_twst, (size_t)(8 * 4096 + 256) * csz, s);
             if (ea == cudaSuccess) ea = pool_alloc((void**)&p.d_dec, (size_t)N * tsz, s);
             if (ea == cudaSuccess) ea = need(&b.red, &b.cred, 8192, s);

@@ -578,6 +578,232 @@ FC2_D void store_tile_blocked(cpx<T>* __restrict__ gout, const cpx<T>* s, SIdx s
     }
 }
 
+// ------------------------------------------------------- double-precision pass
+// Bound by the double pipe (a warp's double instruction takes 64 clocks of its
+// sub-partition), so what counts is the double operations per element:
+//   * every level of every stage is a radix-2 butterfly a +- w b of six fused
+//     operations (three per element and bit), with all of the element's
+//     twiddles in w: a stage of radix Q after passes of radix product D and
+//     stages of product Ns multiplies element n of its butterfly by t^n,
+//     t = e^{2 pi i idx / P}, P = D Ns Q, idx = (j mod D) + D (pp mod Ns) -- the
+//     inter-pass twiddle and the stage twiddle in one -- and level l = 1.. of a
+//     decimation in time needs t^(Q / 2^l) e^{2 pi i k / 2^l}, k < 2^(l-1), half
+//     of them i times the others.  They are read from one table
+//     e^{2 pi i q / M}, q < M / 2 (through L2), each rounded once; forming them
+//     by products took 4 operations each.
+//   * a first pass skips the levels whose second operands are the grid's zero
+//     padding (rows past the occupied ones), in its first two stages;
+//   * a last pass that keeps the centred half of the modes forms only those
+//     outputs of its last level.
+// 73 -> about 50 operations per element for 2^10 x 2^9.  384 grids of 2^19
+// (harmonic counts 2..6): 26.3 -> 16.5 ms for both passes.  The spectra's error
+// against extended-precision sums is unchanged to three digits (2e-15 of the
+// weights at N = 2^12 .. 3e-13 at 2^19, set by the phases).
+template <int Q>
+FC2_D void dit_bfly(cpx<double> a, cpx<double> b, cpx<double> w, cpx<double>* plus,
+                    cpx<double>* minus) {
+    const double px = fma(-b.y, w.y, fma(b.x, w.x, a.x));
+    const double py = fma(b.y, w.x, fma(b.x, w.y, a.y));
+    *plus = mk(px, py);
+    *minus = mk(fma(2.0, a.x, -px), fma(2.0, a.y, -py));
+}
+
+// In-register transform of one butterfly v[0..Q), of which only v[0..MZ) can be
+// nonzero; tw(e) = the table's value for exponent e in units of 1 / P (logP its
+// log2).  TW: twiddles t^n with t = e^{2 pi i idx / P} on element n.  CEN: only
+// outputs k < Q / 4 and k >= 3 Q / 4 are formed.
+template <int QB, int MZ, bool TW, bool CEN, typename Tw>
+FC2_D void dit_stage(cpx<double>* v, int idx, int logP, const Tw& tw) {
+    constexpr int Q = 1 << QB;
+    cpx<double> x[Q], y[Q];
+#pragma unroll
+    for (int n = 0; n < MZ; ++n) x[n] = v[n];
+#pragma unroll
+    for (int l = 1; l <= QB; ++l) {
+        const int N = Q >> l, K = 1 << (l - 1);  // x[k 2N + n] -> y[k N + n], y[(k + K) N + n]
+#pragma unroll
+        for (int kk = 0; kk < (K > 1 ? K / 2 : 1); ++kk) {
+            cpx<double> w = mk(1.0, 0.0);
+            const bool trivial = MZ <= N;  // the second operands are zero
+            if (!trivial) {
+                if constexpr (TW) w = tw(((Q >> l) * idx) + (kk << (logP - l)));
+                else if (l > 2) w = root16<double>(kk * (16 >> l));
+            }
+#pragma unroll
+            for (int half = 0; half < (K > 1 ? 2 : 1); ++half) {
+                const int k = kk + half * (K / 2);  // second half: i w
+#pragma unroll
+                for (int n = 0; n < (N < MZ ? N : MZ); ++n) {
+                    const cpx<double> a = x[k * 2 * N + n];
+                    cpx<double> &p = y[k * N + n], &m = y[(k + K) * N + n];
+                    if (trivial) {
+                        p = a;
+                        m = a;
+                        continue;
+                    }
+                    cpx<double> b = x[k * 2 * N + N + n];
+                    if (half) b = mul_i(b);
+                    if (CEN && l == QB) {  // one output of each last-level butterfly
+                        if (k < Q / 4) {
+                            if (!TW && kk == 0) p = add(a, b);
+                            else p = mk(fma(-b.y, w.y, fma(b.x, w.x, a.x)), fma(b.y, w.x, fma(b.x, w.y, a.y)));
+                        } else {
+                            if (!TW && kk == 0) m = sub(a, b);
+                            else m = mk(fma(b.y, w.y, fma(-b.x, w.x, a.x)), fma(-b.y, w.x, fma(-b.x, w.y, a.y)));
+                        }
+                    } else if (!TW && kk == 0) {
+                        p = add(a, b);
+                        m = sub(a, b);
+                    } else {
+                        dit_bfly<Q>(a, b, w, &p, &m);
+                    }
+                }
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < Q; ++i) x[i] = y[i];
+    }
+#pragma unroll
+    for (int i = 0; i < Q; ++i) v[i] = x[i];
+}
+
+// The pass of k_fft_pass in double: the same tiles, layouts and stages.
+template <int LOGR, int LOGJ, int NT>
+__global__ void __launch_bounds__(NT, 2) k_fft_pass_d(const cpx<double>* __restrict__ in,
+                                                      cpx<double>* __restrict__ out, PassArgs a,
+                                                      const int64_t* __restrict__ Lg,
+                                                      const cpx<double>* __restrict__ twf) {
+    constexpr int R = 1 << LOGR, J = 1 << LOGJ, E = R * J;
+    constexpr int QB1 = stage_bits(LOGR, 0), QB2 = 4, NST = 1 + (LOGR - QB1) / 4;
+    static_assert(QB1 + 4 * (NST - 1) == LOGR && NST >= 2 && NST <= 3, "two or three stages");
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    cpx<double>* s = reinterpret_cast<cpx<double>*>(smem_raw);
+    const int M = 1 << a.logM, S = M >> LOGR;
+    const int g = a.g0 + (int)blockIdx.y;
+    const int j0 = blockIdx.x * J;
+    const cpx<double>* gin = in + (int64_t)g * M;
+    int rows = R;
+    if (a.first) {
+        rows = (int)((Lg[g] + S - 1) / S);
+        if (rows > R) rows = R;
+        for (int e = threadIdx.x; e < E; e += NT) {
+            const int r = e >> LOGJ, jj = e & (J - 1);
+            if (r < rows) cp_elem(&s[phys(e)], &gin[j0 + jj + (int64_t)r * S]);
+            else s[phys(e)] = mk(0.0, 0.0);
+        }
+    } else {
+        const cpx<double>* src = gin + (int64_t)blockIdx.x * E;
+        for (int e = threadIdx.x; e < E; e += NT) cp_elem(&s[phys(e)], &src[e]);
+    }
+    cp_async_wait_all();
+    __syncthreads();
+    const int logD = a.logNs, maskD = (1 << logD) - 1;
+    // one stage of radix 2^QB after 2^DONE; `put` takes each butterfly's outputs
+    auto stage = [&](auto qb_tag, auto done_tag, auto mz_tag, auto tw_tag, auto cen_tag, auto&& put) {
+        constexpr int QB = decltype(qb_tag)::value, DONE = decltype(done_tag)::value;
+        constexpr int MZ = decltype(mz_tag)::value, Q = 1 << QB, NS = 1 << DONE;
+        constexpr int PER = (R / Q) * J / NT;
+        static_assert(PER * NT == (R / Q) * J, "butterflies must divide evenly");
+        const int logP = logD + DONE + QB, sh = a.logM - logP;
+        auto tw = [&](int e) { return __ldg(reinterpret_cast<const double2*>(twf) + ((int64_t)e << sh)); };
+        auto twc = [&](int e) { const double2 z = tw(e); return mk(z.x, z.y); };
+        cpx<double> v[PER][Q];
+#pragma unroll
+        for (int b = 0; b < PER; ++b) {
+            const int bi = threadIdx.x + b * NT, jj = bi % J, pp = bi / J;
+#pragma unroll
+            for (int k = 0; k < MZ; ++k) v[b][k] = s[phys((pp + k * (R / Q)) * J + jj)];
+            const int idx = ((j0 + jj) & maskD) + ((pp & (NS - 1)) << logD);
+            dit_stage<QB, MZ, decltype(tw_tag)::value, decltype(cen_tag)::value>(v[b], idx, logP, twc);
+        }
+        put(v);
+    };
+    // outputs back to the tile: row (pp / Ns) Ns Q + pp mod Ns + k Ns
+    auto to_tile = [&](auto qb_tag, auto done_tag, auto mz_tag, auto tw_tag) {
+        constexpr int QB = decltype(qb_tag)::value, Q = 1 << QB, NS = 1 << decltype(done_tag)::value;
+        stage(qb_tag, done_tag, mz_tag, tw_tag, std::false_type{}, [&](auto& v) {
+            __syncthreads();
+#pragma unroll
+            for (int b = 0; b < (R / Q) * J / NT; ++b) {
+                const int bi = threadIdx.x + b * NT, jj = bi % J, pp = bi / J;
+                const int row = (pp / NS) * NS * Q + (pp & (NS - 1));
+#pragma unroll
+                for (int k = 0; k < Q; ++k) s[phys((row + k * NS) * J + jj)] = v[b][k];
+            }
+            __syncthreads();
+        });
+    };
+    using std::integral_constant;
+    using std::true_type;
+    using B1 = integral_constant<int, QB1>;
+    using B4 = integral_constant<int, 4>;
+    // stage `done` of radix 2^QB with the fewest inputs 2^.. >= kz
+    auto pruned = [&](auto qb_tag, auto done_tag, auto tw_tag, int kz) {
+        constexpr int QB = decltype(qb_tag)::value;
+        if (kz <= 1) to_tile(qb_tag, done_tag, integral_constant<int, 1>{}, tw_tag);
+        else if (QB > 1 && kz <= 2) to_tile(qb_tag, done_tag, integral_constant<int, 2>{}, tw_tag);
+        else if (QB > 2 && kz <= 4) to_tile(qb_tag, done_tag, integral_constant<int, (QB > 1 ? 4 : 2)>{}, tw_tag);
+        else if (QB > 3 && kz <= 8) to_tile(qb_tag, done_tag, integral_constant<int, (QB > 2 ? 8 : 2)>{}, tw_tag);
+        else to_tile(qb_tag, done_tag, integral_constant<int, (1 << QB)>{}, tw_tag);
+    };
+    auto last_put = [&](auto& v) {  // modes straight from registers
+        const int jj = threadIdx.x % J, pp = threadIdx.x / J;
+#pragma unroll
+        for (int k = 0; k < 16; ++k) {
+            const int o = j0 + jj + ((pp + k * (R / 16)) << logD);
+            const int m = (o < M / 2) ? o : o - M;
+            store_mode<double>(out, a, g, m, v[0][k]);
+        }
+    };
+    auto last_put_centred = [&](auto& v) {
+        const int jj = threadIdx.x % J, pp = threadIdx.x / J;
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            const int k = q < 4 ? q : q + 8;
+            const int o = j0 + jj + ((pp + k * (R / 16)) << logD);
+            const int m = (o < M / 2) ? o : o - M;
+            store_mode<double>(out, a, g, m, v[0][k]);
+        }
+    };
+    using DL = integral_constant<int, LOGR - 4>;
+    using Full = integral_constant<int, 16>;
+    if (a.first) {  // no inter-pass twiddle; zero rows pruned
+        const int kz1 = (rows + (R >> QB1) - 1) >> (LOGR - QB1);
+        pruned(B1{}, integral_constant<int, 0>{}, std::false_type{}, kz1);
+        // with one nonzero input per butterfly, stage 1's outputs fill rows
+        // below rows 2^QB1
+        const int kz2 = kz1 > 1 ? 16 : ((rows << QB1) + (R >> 4) - 1) >> (LOGR - 4);
+        pruned(B4{}, B1{}, true_type{}, kz2);
+        if constexpr (NST == 3) to_tile(B4{}, integral_constant<int, QB1 + 4>{}, Full{}, true_type{});
+    } else {
+        to_tile(B1{}, integral_constant<int, 0>{}, integral_constant<int, (1 << QB1)>{}, true_type{});
+        if constexpr (NST == 3) to_tile(B4{}, B1{}, Full{}, true_type{});
+        if (a.last) {
+            // modes |m| <= M / 4 are outputs k < 4 and k >= 12 of the last stage,
+            // whose step is M / 16
+            if (2 * (int64_t)a.N <= M) stage(B4{}, DL{}, Full{}, true_type{}, true_type{}, last_put_centred);
+            else stage(B4{}, DL{}, Full{}, true_type{}, std::false_type{}, last_put);
+            return;
+        }
+        to_tile(B4{}, DL{}, Full{}, true_type{});
+    }
+    cpx<double>* gout = out + (int64_t)g * M;
+    const int LOGJn = a.logJn, logBlk = a.logRn + a.logJn;
+    if (logD == 0 && a.logM - a.logRn == LOGR) {
+        for (int e = threadIdx.x; e < E; e += NT) {
+            const TileElem te = tile_elem(e, LOGJn, LOGJ);
+            gout[rowcol_pos(te.k, j0 + te.jj, LOGJn, logBlk)] = s[phys(te.k * J + te.jj)];
+        }
+    } else {
+        const int logSn = a.logM - a.logRn;
+        for (int e = threadIdx.x; e < E; e += NT) {
+            const TileElem te = tile_elem(e, LOGJn, LOGJ);
+            const int64_t i = stockham_out(j0 + te.jj, te.k, logD, LOGR);
+            gout[blocked_pos(i, logSn, LOGJn, logBlk)] = s[phys(te.k * J + te.jj)];
+        }
+    }
+}
+
 // ------------------------------------------------- pruned small transform
 // Q-point DFT (sign +) of v when only v[0..MZ) can be nonzero: with
 // k = (Q/MZ) k1 + k2, X_k = sum_{n<MZ} (v_n w_Q^{n k2}) w_MZ^{n k1}, i.e. Q/MZ
@@ -1232,9 +1458,29 @@ static bool r32_pass(int family, int logR) {
     return (family == FFT_R32 && logR == 10) || (family == FFT_R32X && (logR == 9 || logR == 10));
 }
 
+// fp32: tiles of 2^13 complex (64 KB), radix <= 2^12; fp64: 2^12 (64 KB), <= 2^11.
+template <typename T> struct FftCfg;
+template <> struct FftCfg<float> { static constexpr int LOGE = 13; static constexpr int NT = 512; static constexpr int MAXR = 12; };
+template <> struct FftCfg<double> { static constexpr int LOGE = 12; static constexpr int NT = 256; static constexpr int MAXR = 11; };
+
+// Two-level table split: entries of the low and high parts.  The fused double
+// passes keep the whole table q < M / 2 in the low part.
+void twiddle_split(int logM, bool fused, int* sh, int64_t* nlo, int64_t* nhi) {
+    if (fused && logM > FftCfg<double>::MAXR) {
+        *sh = logM - 1;
+        *nlo = 1ll << *sh;
+        *nhi = 1;
+        return;
+    }
+    *sh = (logM + 1) / 2;
+    *nlo = 1ll << *sh;
+    *nhi = (1ll << logM) >> *sh;
+}
+
 cudaError_t init_twiddles(fc2_plan_s* p, cudaStream_t s) {
-    int sh = (p->logM + 1) / 2;
-    int64_t nlo = 1ll << sh, nhi = p->M >> sh;
+    int sh;
+    int64_t nlo, nhi;
+    twiddle_split(p->logM, p->fused_fft, &sh, &nlo, &nhi);
     p->tw_shift = sh;
     int64_t nmax = std::max(nlo, nhi);
     unsigned blocks = (unsigned)((nmax + 255) / 256);
@@ -1277,10 +1523,6 @@ cudaError_t init_twiddles(fc2_plan_s* p, cudaStream_t s) {
 }
 
 // -------------------------------------------------------------- pass plan
-// fp32: tiles of 2^13 complex (64 KB), radix <= 2^12; fp64: 2^12 (64 KB), <= 2^11.
-template <typename T> struct FftCfg;
-template <> struct FftCfg<float> { static constexpr int LOGE = 13; static constexpr int NT = 512; static constexpr int MAXR = 12; };
-template <> struct FftCfg<double> { static constexpr int LOGE = 12; static constexpr int NT = 256; static constexpr int MAXR = 11; };
 
 void plan_fft_passes(fc2_plan_s* p) {
     const int maxr = p->fp64 ? FftCfg<double>::MAXR : FftCfg<float>::MAXR;
@@ -1596,6 +1838,20 @@ static cudaError_t run_pass(fc2_plan_s* p, const void* in, void* out, const Pass
     return cudaGetLastError();
 }
 
+template <int LOGR>
+static cudaError_t run_pass_d(fc2_plan_s* p, const void* in, void* out, const PassArgs& a,
+                              cudaStream_t s) {
+    constexpr int LOGJ = FftCfg<double>::LOGE - LOGR, NT = FftCfg<double>::NT;
+    constexpr size_t smem = (size_t)(phys((1 << FftCfg<double>::LOGE) - 1) + 1) * sizeof(cpx<double>);
+    auto kern = k_fft_pass_d<LOGR, LOGJ, NT>;
+    const cudaError_t e = raise_smem_limit((const void*)kern, smem);
+    if (e != cudaSuccess) return e;
+    dim3 grid((unsigned)((p->M >> LOGR) >> LOGJ), (unsigned)a.ng);
+    kern<<<grid, NT, smem, s>>>((const cpx<double>*)in, (cpx<double>*)out, a, p->d_L,
+                                (const cpx<double>*)p->d_twlo);
+    return cudaGetLastError();
+}
+
 template <int RB, int LOGR>
 static cudaError_t run_pass64(fc2_plan_s* p, const void* in, void* out, const PassArgs& a,
                               cudaStream_t s) {
@@ -1667,6 +1923,14 @@ static cudaError_t run_radix(fc2_plan_s* p, const void* in, void* out, const Pas
         return cudaErrorInvalidValue;
     }
     constexpr int LOGJ = FftCfg<T>::LOGE - LOGR;
+    // Batches return float, where the fused kernel's other rounding is far below
+    // an ulp; a plan returns double Delta chi^2, and its bins of coefficient norm
+    // up to 1e7 would carry a change of rounding to 3e-7 of the rms, so plans keep
+    // the operation order of k_fft_pass (the fused kernel would take a
+    // 2^20-bin plan of four harmonics from 6.5 to 5.2 ms).
+    if constexpr (sizeof(T) == 8 && LOGJ >= 0) {
+        if (p->fused_fft) return run_pass_d<LOGR>(p, in, out, a, s);
+    }
     if constexpr (LOGJ >= 0) return run_pass<T, LOGR, LOGJ, FftCfg<T>::NT>(p, in, out, a, s);
     return cudaErrorInvalidValue;
 }
@@ -1788,6 +2052,21 @@ static int replay_plan(int logM, bool fp64, int family, const std::vector<int>& 
                 } else if (sh.kind == PK_BULK && bulk_stage1_bits(LOGR) == 5) {
                     // radix-32 stage 1: t0 up to (R/16 - 1) jm, steps (R/32) jm x 1, 4, 16
                     qmax = std::max<int64_t>(((R / 16 - 1) * jmax) << lts, ((R / 32) * 16 * jmax) << lts);
+                } else if (fp64) {
+                    // k_fft_pass_d (batches): level 1 of each stage reaches (Q / 2) idx, idx < P / Q,
+                    // P <= D R, in a table of M / 2 entries
+                    for (int done = 0; done < LOGR; done += stage_bits(LOGR, done)) {
+                        const int qb = stage_bits(LOGR, done), logP = logNs + done + qb;
+                        const int64_t idx = jmax + (((1ll << done) - 1) << logNs);
+                        qmax = std::max<int64_t>(qmax, (idx << (qb - 1)) << (logM - logP));
+                        for (int l = 2; l <= qb; ++l)
+                            qmax = std::max<int64_t>(
+                                qmax, ((idx << (qb - l)) + (((1ll << (l - 2)) - 1) << (logP - l)))
+                                          << (logM - logP));
+                    }
+                    if (qmax >= M / 2) return fail(pi, 3, bx, qmax);
+                    const int Q1 = 1 << stage_bits(LOGR, 0);  // k_fft_pass
+                    qmax = std::max<int64_t>(((R / Q1 - 1) * jmax) << lts, ((R / Q1) * jmax) << lts);
                 } else {
                     const int Q1 = 1 << stage_bits(LOGR, 0);
                     qmax = std::max<int64_t>(((R / Q1 - 1) * jmax) << lts, ((R / Q1) * jmax) << lts);
