@@ -1098,7 +1098,7 @@ __global__ void __launch_bounds__(P32_NT, 1) k_fft_pass32(const cpx<float>* __re
 }
 
 // ------------------------------------------- radix-16 pass fed by bulk copies
-// Float passes of radix R = 2^8..2^12 as the in-CTA Stockham stages of
+// Float passes of radix R = 2^10..2^12 as the in-CTA Stockham stages of
 // k_fft_pass (radix 16; the first stage takes LOGR mod 4 bits when that is
 // nonzero), on tiles of 8192 elements with one persistent 512-thread CTA per
 // SM.  A later pass reads each tile -- one contiguous 64 KB run of the blocked
@@ -1175,9 +1175,8 @@ FC2_D void dft16_centred(cpx<T>* v) {
     for (int k = 4; k < 8; ++k) v[k + 8] = sub(e[k], k == 4 ? mul_i(o[4]) : mul(o[k], root16<T>(k)));
 }
 
-// First-stage radix bits of the bulk-copy pass: radix 32 for 2^9 passes (two
-// stages, 32 x 16: the first with half the threads, one butterfly of 32
-// each), else as the other shared-memory stages (2^9 would otherwise take
+// First-stage radix bits of the bulk-copy passes: radix 32 for 2^9 (two stages,
+// 32 x 16), else as the other shared-memory stages (2^9 would otherwise take
 // 2 x 16 x 16, one more pass through shared memory).
 FC2_HD constexpr int bulk_stage1_bits(int LOGR) { return LOGR == 9 ? 5 : stage_bits(LOGR, 0); }
 
@@ -1202,17 +1201,14 @@ __global__ void __launch_bounds__(PT_NT, 1) k_fft_pass_tma(const cpx<float>* __r
     constexpr int NT = PT_NT;
     constexpr int NST = stage_tw_size(LOGR);
     constexpr int NWK = phys(E - 1) + 1;
-    static_assert(LOGR >= 8 && LOGR <= 12, "radix 2^8..2^12");
+    static_assert(LOGR >= 10 && LOGR <= 12, "radix 2^10..2^12 (k_fft_pass_duo: 2^8, 2^9)");
     // stage 1 (radix Q1), middle stages of radix 16, last stage of radix 16
     constexpr int QB1 = bulk_stage1_bits(LOGR), Q1 = 1 << QB1;
     constexpr int NB1 = (R / Q1) * J;                      // stage-1 butterflies
-    constexpr bool HALF1 = NB1 < NT;                       // threads tid >= NB1 idle in stage 1
-    constexpr int PER1 = HALF1 ? 1 : NB1 / NT;
+    constexpr int PER1 = NB1 / NT;
     constexpr int DL = LOGR - 4, NSL = 1 << DL;            // last stage: Ns = R / 16
     constexpr int TOFF_L = NST - 15 * NSL;                 // its twiddle table
-    static_assert(HALF1 ? (NT % NB1 == 0 && Q1 == 32) : PER1 * NT == NB1,
-                  "stage-1 butterflies must divide evenly");
-    static_assert(Q1 <= 32, "stage-1 radix");
+    static_assert(PER1 * NT == NB1, "stage-1 butterflies must divide evenly");
     static_assert(NSL * J == NT, "one last-stage butterfly per thread");
     extern __shared__ __align__(16) unsigned char smem_raw[];
     cpx<T>* ib = reinterpret_cast<cpx<T>*>(smem_raw);  // [2][E] input buffers
@@ -1260,11 +1256,7 @@ __global__ void __launch_bounds__(PT_NT, 1) k_fft_pass_tma(const cpx<float>* __r
     // and tile, the second factor (and the step w^{(R/Q1) jm 2^lts}) one lookup per
     // (column, b) and tile, kept in shared memory -- instead of two lookups per
     // butterfly.
-    // (a radix-32 stage 1: per column the powers step^q, q = 1, 2, 3, 4, 8,
-    // 12, 16 of step = w^{(R/Q1) jm 2^lts}, each a table lookup; element k's
-    // factor is t0 step^(k mod 4) step^(4 ((k >> 2) mod 4)) step^(16 (k >> 4)),
-    // three products of looked-up values)
-    constexpr int TW1 = HALF1 ? 7 : PER1 + 1;
+    constexpr int TW1 = PER1 + 1;
     __shared__ cpx<T> tw1[J * TW1];
     cpx<T> t0 = mk<T>(1.f, 0.f);
     for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++it) {
@@ -1279,9 +1271,7 @@ __global__ void __launch_bounds__(PT_NT, 1) k_fft_pass_tma(const cpx<float>* __r
             for (int q = tid; q < J * TW1; q += NT) {
                 const int cj = q / TW1, bb = q - cj * TW1;
                 const int jm = (j0 + cj) & nsg_mask;
-                int64_t e;
-                if constexpr (HALF1) e = (int64_t)(R / Q1) * jm * (bb < 3 ? bb + 1 : 4 * (bb - 2));
-                else e = (bb < PER1) ? (int64_t)bb * (R / 16) * jm : (int64_t)(R / Q1) * jm;
+                const int64_t e = (bb < PER1) ? (int64_t)bb * (R / 16) * jm : (int64_t)(R / Q1) * jm;
                 tw1[q] = twiddle(twlo, twhi, a.tws, e << lts);
             }
             const int jm = (j0 + (tid & (J - 1))) & nsg_mask;
@@ -1313,7 +1303,6 @@ __global__ void __launch_bounds__(PT_NT, 1) k_fft_pass_tma(const cpx<float>* __r
 #pragma unroll
             for (int b = 0; b < PER1; ++b) {
                 const int bi = tid + b * NT;
-                if (HALF1 && bi >= NB1) break;
                 const int jj = bi & (J - 1), pp = bi >> LOGJ;
                 cpx<T> v[Q1];
                 if (!bulk) {
@@ -1326,23 +1315,7 @@ __global__ void __launch_bounds__(PT_NT, 1) k_fft_pass_tma(const cpx<float>* __r
 #pragma unroll
                     for (int k = 0; k < Q1; ++k) v[k] = src[(pp + k * (R / Q1)) * J + jj];
                     const int jm = (j0 + jj) & nsg_mask;
-                    if constexpr (HALF1) {
-                        if (logNs > 0 && jm != 0) {
-                            // w_M^{(pp + k R/Q1) jm 2^lts} = t0 step^(k & 3) step^(k & 12) step^(k & 16)
-                            const cpx<T>* sq = tw1 + jj * TW1;  // step^1, 2, 3, 4, 8, 12, 16
-                            cpx<T> lo[4];
-                            lo[0] = t0;
-#pragma unroll
-                            for (int q = 1; q < 4; ++q) lo[q] = mul(t0, sq[q - 1]);
-#pragma unroll
-                            for (int k = 0; k < Q1; ++k) {
-                                cpx<T> w = lo[k & 3];
-                                if (((k >> 2) & 3) != 0) w = mul(w, sq[2 + ((k >> 2) & 3)]);
-                                if ((k >> 4) != 0) w = mul(w, sq[6]);
-                                v[k] = mul(v[k], w);
-                            }
-                        }
-                    } else if (logNs > 0 && jm != 0) {
+                    if (logNs > 0 && jm != 0) {
                         // w_M^{(pp + k R/Q1) jm 2^lts} = base * step^k, step^k = lo[k & 3] hi[k >> 2]
                         const cpx<T> base = mul(t0, tw1[jj * TW1 + b]);
                         const cpx<T> st1 = tw1[jj * TW1 + PER1];
@@ -1449,6 +1422,334 @@ __global__ void __launch_bounds__(PT_NT, 1) k_fft_pass_tma(const cpx<float>* __r
             store_tile_blocked<LOGR, LOGJ, NT>(out + (int64_t)g * M, wk,
                                                [](int e) { return phys(e); }, j0, a, tid);
             __syncthreads();
+        }
+    }
+}
+
+// ------------------------------------------- the 2^8 and 2^9 bulk-copy passes
+// The passes of radix 2^8 and 2^9 with the stages and arithmetic of
+// k_fft_pass_tma (16 x 16 and 32 x 16; results are bit-equal), by two groups of
+// 256 threads per SM, each on a tile of its own.  A transform of one tile is a
+// chain -- wait for its copy, stage 1, barrier, last stage, store -- and with
+// one tile per SM in lockstep each link idles what the others need (issue
+// active 54%, and the 32 x 16 pass's 256 first butterflies left half of 512
+// threads waiting); two chains out of step fill each other's gaps.  A group
+// transforms in place: its 64 KB buffer receives the tile by bulk copies, holds
+// the exchange between the stages, and is handed back to the copy engine as soon
+// as the last stage has read it, so the next tile arrives during the last
+// stage's arithmetic and stores.  Lanes run along the columns (a half-warp per
+// 128-byte row), free of bank conflicts without padding.  Results on the way
+// to another pass are staged through the buffer (columns XORed with the row) and
+// leave in runs of the next pass's layout.  A first pass skips the butterfly
+// levels whose second operands are zero padding; a middle pass before the last
+// one stores straight from registers, contiguous along the columns.
+// Bound by memory: the later passes run at 6.0-6.1 TB/s, 0.88 of the copy rate.
+//   1024 survey curves, second pass 2^9:  17.7 -> 12.95 ms
+//   24 grids of 2^26: both 2^9 passes 18.0 -> 3.6 + 4.2 ms (the middle one 10.7
+//     with its results staged), last 2^8 4.2 -> 3.2 ms
+//   1536 grids of 2^17: first 2^9 1.25 -> 0.64, last 2^8 0.48 -> 0.39 ms
+constexpr int DUO_GT = 256;                  // threads of a group
+constexpr int DUO_NT = 2 * DUO_GT;
+
+FC2_D void duo_sync(int g) { asm volatile("bar.sync %0, 256;\n" ::"r"(g + 1) : "memory"); }
+FC2_D bool duo_sync_and(int g, bool ok) {
+    uint32_t r;
+    asm volatile(
+        "{\n .reg .pred p, q;\n setp.ne.u32 p, %2, 0;\n bar.red.and.pred q, %1, 256, p;\n"
+        " selp.u32 %0, 1, 0, q;\n}\n"
+        : "=r"(r)
+        : "r"(g + 1), "r"((uint32_t)ok)
+        : "memory");
+    return r != 0;
+}
+
+// SmallDFT<T, Q> of v when only v[0..MZ) can be nonzero: the same operations
+// without those on the zeros.
+template <typename T, int Q, int MZ>
+struct ZeroDFT {
+    static FC2_D void run(cpx<T>* v) {
+        if constexpr (MZ == Q) {
+            SmallDFT<T, Q>::run(v);
+        } else if constexpr (MZ == 1) {
+#pragma unroll
+            for (int k = 1; k < Q; ++k) v[k] = v[0];
+        } else {
+            cpx<T> e[Q / 2], o[Q / 2];
+#pragma unroll
+            for (int i = 0; i < MZ / 2; ++i) { e[i] = v[2 * i]; o[i] = v[2 * i + 1]; }
+            ZeroDFT<T, Q / 2, MZ / 2>::run(e);
+            ZeroDFT<T, Q / 2, MZ / 2>::run(o);
+#pragma unroll
+            for (int k = 0; k < Q / 2; ++k) {
+                cpx<T> t;
+                if (k == 0) t = o[k];
+                else if (4 * k == Q) t = mul_i(o[k]);
+                else if constexpr (Q <= 16) t = mul(o[k], root16<T>(k * (16 / Q)));
+                else t = mul(o[k], root64<T>(k * (64 / Q)));
+                v[k] = add(e[k], t);
+                v[k + Q / 2] = sub(e[k], t);
+            }
+        }
+    }
+};
+
+template <int LOGR>
+constexpr size_t pass_duo_smem() {
+    constexpr int TW1 = LOGR == 9 ? 7 : 1;
+    return (size_t)(2 * (1 << PT_LOGE) + stage_tw_size(LOGR) + 2 * ((1 << PT_LOGE) >> LOGR) * TW1) *
+               sizeof(cpx<float>) +
+           2 * sizeof(uint64_t);
+}
+
+template <int LOGR, bool FIRST>
+__global__ void __launch_bounds__(DUO_NT, 1) k_fft_pass_duo(const cpx<float>* __restrict__ in,
+                                                         cpx<float>* __restrict__ out, PassArgs a,
+                                                         const int64_t* __restrict__ Lg,
+                                                         const cpx<float>* __restrict__ twlo,
+                                                         const cpx<float>* __restrict__ twhi,
+                                                         const cpx<float>* __restrict__ twst, int G,
+                                                         int* __restrict__ status,
+                                                         long long wait_cycles, int drop_tile) {
+    using T = float;
+    constexpr int R = 1 << LOGR, LOGJ = PT_LOGE - LOGR, J = 1 << LOGJ, E = 1 << PT_LOGE;
+    constexpr int NST = stage_tw_size(LOGR);
+    static_assert(LOGR == 8 || LOGR == 9, "radix 2^8 or 2^9");
+    constexpr int QB1 = bulk_stage1_bits(LOGR), Q1 = 1 << QB1;
+    constexpr int PERB = (R / Q1) * J / DUO_GT;      // stage-1 butterflies per thread
+    constexpr int NSL = R / 16, TOFF_L = NST - 15 * NSL;
+    static_assert(PERB * Q1 == 32 && NSL * J == 2 * DUO_GT, "32 elements per thread");
+    constexpr int TW1 = LOGR == 9 ? 7 : 1;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int grp = threadIdx.x / DUO_GT, gt = threadIdx.x % DUO_GT;
+    cpx<T>* bufs = reinterpret_cast<cpx<T>*>(smem_raw);
+    cpx<T>* buf = bufs + grp * E;
+    cpx<T>* st = bufs + 2 * E;
+    cpx<T>* tw1 = st + NST + grp * J * TW1;
+    uint64_t* mbar = reinterpret_cast<uint64_t*>(st + NST + 2 * J * TW1) + grp;
+    const int M = 1 << a.logM, S = M >> LOGR;
+    const int tiles_x = S >> LOGJ, ntiles = tiles_x * G;
+    for (int i = threadIdx.x; i < NST; i += DUO_NT) st[i] = twst[i];
+    if (!FIRST && gt == 0) {
+        mbar_init(mbar, 1);
+        mbar_init_fence();
+    }
+    __syncthreads();
+    // a group's thread 0: copy tile t into its buffer (four 16 KB pieces, one
+    // mbarrier); drop_tile >= 0, a fault-injection setting of the tests: that
+    // tile's barrier is armed but its copy is never issued, so its wait runs out
+    auto issue = [&](int t) {
+        const int gtl = t / tiles_x, bt = t - gtl * tiles_x;
+        const cpx<T>* src = in + (int64_t)(a.g0 + gtl) * M + (int64_t)bt * E;
+        mbar_expect_tx(mbar, (unsigned)(E * sizeof(cpx<T>)));
+        if (t == drop_tile) return;
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+            bulk_g2s(buf + c * (E / 4), src + c * (E / 4), (unsigned)(E / 4 * sizeof(cpx<T>)), mbar);
+    };
+    const int tile0 = blockIdx.x * 2 + grp, tstep = 2 * (int)gridDim.x;
+    if (!FIRST && gt == 0 && tile0 < ntiles) issue(tile0);
+    const int logNs = a.logNs, nsg_mask = (1 << logNs) - 1, lts = a.logM - logNs - LOGR;
+    const bool same_radix = logNs == 0 && a.logM - a.logRn == LOGR;
+    // a middle pass before the last one: output k of column j = jh Ns + jl is
+    // column jl + k Ns of the last pass, row jh -- contiguous along jl, so the
+    // lanes' runs of columns go straight from registers
+    const bool mid = !a.last && logNs + LOGR + a.logRn == a.logM && logNs >= a.logJn && logNs >= LOGJ;
+    int it = 0;
+    for (int tile = tile0; tile < ntiles; tile += tstep, ++it) {
+        const int gl = tile / tiles_x, g = a.g0 + gl, bx = tile - gl * tiles_x, j0 = bx * J;
+        cpx<T> v[32], t0[PERB];
+        // inter-pass twiddles as k_fft_pass_tma's: t0 per butterfly, and per column
+        // the step's powers 1, 2, 3, 4, 8, 12, 16 (2^9) or the step (2^8)
+        if constexpr (!FIRST) {
+            for (int q = gt; q < J * TW1; q += DUO_GT) {
+                const int cj = q / TW1, bb = q - cj * TW1;
+                const int jm = (j0 + cj) & nsg_mask;
+                const int64_t e = (int64_t)(R / Q1) * jm * (bb < 3 ? bb + 1 : 4 * (bb - 2));
+                tw1[q] = twiddle(twlo, twhi, a.tws, e << lts);
+            }
+#pragma unroll
+            for (int b = 0; b < PERB; ++b) {
+                const int bi = gt + b * DUO_GT;
+                const int jm = (j0 + (bi & (J - 1))) & nsg_mask;
+                t0[b] = twiddle(twlo, twhi, a.tws, (int64_t)((bi >> LOGJ) * jm) << lts);
+            }
+            const bool ok = mbar_wait_bounded(mbar, (unsigned)(it & 1), wait_cycles);
+            if (!duo_sync_and(grp, ok)) {
+                // give up: report, then wait (again bounded) for the group's one copy
+                // in flight so that none is left writing into an exited CTA
+                if (gt == 0 && status) atomicExch(status, (int)FC2_ERR_TIMEOUT);
+                mbar_wait_bounded(mbar, (unsigned)(it & 1), wait_cycles);
+                return;
+            }
+        }
+        // ---- stage 1: radix Q1, rows pp + k R / Q1 -> rows pp Q1 + k
+        if constexpr (FIRST) {
+            const cpx<T>* gin = in + (int64_t)g * M;
+            int rows = (int)((Lg[g] + S - 1) / S);
+            if (rows > R) rows = R;
+            auto first = [&](auto mz_tag) {
+                constexpr int MZ = decltype(mz_tag)::value;
+#pragma unroll
+                for (int b = 0; b < PERB; ++b) {
+                    const int bi = gt + b * DUO_GT, jj = bi & (J - 1), pp = bi >> LOGJ;
+#pragma unroll
+                    for (int k = 0; k < MZ; ++k) {
+                        const int r = pp + k * (R / Q1);
+                        v[b * Q1 + k] = (r < rows) ? gin[j0 + jj + (int64_t)r * S] : mk<T>(0.f, 0.f);
+                    }
+                    ZeroDFT<T, Q1, MZ>::run(v + b * Q1);
+                }
+            };
+            const int kz = (rows + R / Q1 - 1) / (R / Q1);
+            if (kz <= 2) first(std::integral_constant<int, 2>{});
+            else if (kz <= 4) first(std::integral_constant<int, 4>{});
+            else if (kz <= 8) first(std::integral_constant<int, 8>{});
+            else if (kz <= 16) first(std::integral_constant<int, 16>{});
+            else first(std::integral_constant<int, Q1>{});
+        } else {
+#pragma unroll
+            for (int b = 0; b < PERB; ++b) {
+                const int bi = gt + b * DUO_GT, jj = bi & (J - 1), pp = bi >> LOGJ;
+                cpx<T>* u = v + b * Q1;
+#pragma unroll
+                for (int k = 0; k < Q1; ++k) u[k] = buf[(pp + k * (R / Q1)) * J + jj];
+                if (((j0 + jj) & nsg_mask) != 0) {
+                    const cpx<T>* sq = tw1 + jj * TW1;
+                    if constexpr (LOGR == 9) {
+                        // t0 step^(k & 3) step^(k & 12) step^(k & 16)
+                        cpx<T> lo[4];
+                        lo[0] = t0[b];
+#pragma unroll
+                        for (int q = 1; q < 4; ++q) lo[q] = mul(t0[b], sq[q - 1]);
+#pragma unroll
+                        for (int k = 0; k < Q1; ++k) {
+                            cpx<T> w = lo[k & 3];
+                            if (((k >> 2) & 3) != 0) w = mul(w, sq[2 + ((k >> 2) & 3)]);
+                            if ((k >> 4) != 0) w = mul(w, sq[6]);
+                            u[k] = mul(u[k], w);
+                        }
+                    } else {
+                        // base step^k, step^k = lo[k & 3] hi[k >> 2]
+                        const cpx<T> st1 = sq[0];
+                        cpx<T> lo[4], hi[4];
+                        lo[1] = st1;
+                        lo[2] = mul(st1, st1);
+                        lo[3] = mul(lo[2], st1);
+                        hi[1] = mul(lo[2], lo[2]);
+                        hi[2] = mul(hi[1], hi[1]);
+                        hi[3] = mul(hi[2], hi[1]);
+#pragma unroll
+                        for (int k = 0; k < Q1; ++k) {
+                            cpx<T> w = t0[b];
+                            if ((k & 3) != 0) w = mul(w, lo[k & 3]);
+                            if ((k >> 2) != 0) w = mul(w, hi[k >> 2]);
+                            u[k] = mul(u[k], w);
+                        }
+                    }
+                }
+                SmallDFT<T, Q1>::run(u);
+            }
+            duo_sync(grp);  // the group has read the buffer
+        }
+#pragma unroll
+        for (int b = 0; b < PERB; ++b) {
+            const int bi = gt + b * DUO_GT, jj = bi & (J - 1), pp = bi >> LOGJ;
+#pragma unroll
+            for (int k = 0; k < Q1; ++k) buf[(pp * Q1 + k) * J + jj] = v[b * Q1 + k];
+        }
+        duo_sync(grp);
+        // ---- last stage (radix 16, Ns = R / 16): two butterflies per thread
+#pragma unroll
+        for (int b = 0; b < 2; ++b) {
+            const int bi = gt + b * DUO_GT, jj = bi & (J - 1), pp = bi >> LOGJ;
+#pragma unroll
+            for (int k = 0; k < 16; ++k) v[b * 16 + k] = buf[(pp + k * NSL) * J + jj];
+        }
+        duo_sync(grp);  // the buffer is free
+        const int next = tile + tstep;
+        if (!FIRST && (a.last || mid) && gt == 0 && next < ntiles) {
+            fence_proxy_async_smem();
+            issue(next);
+        }
+        const bool centred = a.last && g >= a.npk && 2 * a.N == M && 2 * a.hN == a.N &&
+                             16 * (NSL << logNs) == M;
+#pragma unroll
+        for (int b = 0; b < 2; ++b) {
+            const int bi = gt + b * DUO_GT, jj = bi & (J - 1), pp = bi >> LOGJ;
+            cpx<T>* u = v + b * 16;
+#pragma unroll
+            for (int k = 1; k < 16; ++k) u[k] = mul(u[k], st[TOFF_L + (k - 1) * NSL + pp]);
+            if (!FIRST && centred) {
+                dft16_centred(u);
+                const int o0 = j0 + jj + (pp << logNs), step = NSL << logNs;
+                cpx<T>* spec = out + (int64_t)(a.npk + g) * a.N;
+#pragma unroll
+                for (int k = 0; k < 4; ++k) spec[o0 + k * step + a.hN] = u[k];
+#pragma unroll
+                for (int k = 12; k < 16; ++k) spec[o0 + k * step - (M - a.hN)] = u[k];
+                continue;
+            }
+            SmallDFT<T, 16>::run(u);
+            if (!FIRST && a.last) {
+                const int o0 = j0 + jj + (pp << logNs), step = NSL << logNs;
+                if (g < a.npk) {
+                    cpx<T>* plus = out + (int64_t)(2 * g) * a.N;
+                    cpx<T>* minus = plus + a.N;
+#pragma unroll
+                    for (int k = 0; k < 16; ++k) {
+                        const int o = o0 + k * step;
+                        const int jp = o - a.sh;
+                        const int jmi = ((M - o) & (M - 1)) - a.sh;
+                        if ((unsigned)jp < (unsigned)a.N) plus[jp] = u[k];
+                        if ((unsigned)jmi < (unsigned)a.N) minus[jmi] = u[k];
+                    }
+                } else {
+                    cpx<T>* spec = out + (int64_t)(a.npk + g) * a.N;
+                    const int lo_end = a.N - a.hN, hi_start = M - a.hN;
+#pragma unroll
+                    for (int k = 0; k < 16; ++k) {
+                        const int o = o0 + k * step;
+                        if (o < lo_end) spec[o + a.hN] = u[k];
+                        else if (o >= hi_start) spec[o - hi_start] = u[k];
+                    }
+                }
+            } else if (!FIRST && mid) {
+                const int LOGJn = a.logJn, logBlk = a.logRn + a.logJn;
+                const int jl = (j0 + jj) & nsg_mask, jh = (j0 + jj) >> logNs;
+                const int up = logNs - LOGJn;  // rows to tiles
+                cpx<T>* dst = out + (int64_t)g * M + ((int64_t)((jl >> LOGJn) + (pp << up)) << logBlk) +
+                              (jh << LOGJn) + (jl & ((1 << LOGJn) - 1));
+                const int64_t step = (int64_t)(NSL << up) << logBlk;
+#pragma unroll
+                for (int k = 0; k < 16; ++k) dst[k * step] = u[k];
+            } else {
+#pragma unroll
+                for (int k = 0; k < 16; ++k) {
+                    const int row = pp + k * NSL;
+                    buf[row * J + (jj ^ (row & (J - 1)))] = u[k];
+                }
+            }
+        }
+        if (FIRST || !(a.last || mid)) {
+            duo_sync(grp);
+            cpx<T>* gout = out + (int64_t)g * M;
+            auto slot = [](int e) { return e ^ ((e >> LOGJ) & (J - 1)); };
+            if (same_radix) {
+                // two-pass plan: logical output j R + k is column k, row j of the last pass
+                const int LOGJn = a.logJn, logBlk = a.logRn + a.logJn;
+#pragma unroll 8
+                for (int e = gt; e < E; e += DUO_GT) {
+                    const TileElem te = tile_elem(e, LOGJn, LOGJ);
+                    gout[rowcol_pos(te.k, j0 + te.jj, LOGJn, logBlk)] = buf[slot(te.k * J + te.jj)];
+                }
+            } else {
+                store_tile_blocked<LOGR, LOGJ, DUO_GT>(gout, buf, slot, j0, a, gt);
+            }
+            duo_sync(grp);
+            if (!FIRST && gt == 0 && next < ntiles) {
+                fence_proxy_async_smem();
+                issue(next);
+            }
         }
     }
 }
@@ -1569,7 +1870,7 @@ static PassShape pass_shape(int logM, bool fp64, int family, int logR) {
     if (!fp64 && r32_pass(family, logR))
         return PassShape{PK_R32, P64_LOGE, P64_LOGE - logR, P32_NT};
     if (!fp64 && family != FFT_R16 && logR >= 8 && logR <= 12)
-        return PassShape{PK_BULK, PT_LOGE, PT_LOGE - logR, PT_NT};
+        return PassShape{PK_BULK, PT_LOGE, PT_LOGE - logR, logR <= 9 ? DUO_GT : PT_NT};
     const int loge = fp64 ? FftCfg<double>::LOGE : FftCfg<float>::LOGE;
     return PassShape{PK_R16, loge, loge - logR, fp64 ? FftCfg<double>::NT : FftCfg<float>::NT};
 }
@@ -1882,6 +2183,24 @@ static cudaError_t run_pass64(fc2_plan_s* p, const void* in, void* out, const Pa
 }
 
 template <int LOGR>
+static cudaError_t run_pass_duo(fc2_plan_s* p, const void* in, void* out, const PassArgs& a,
+                                cudaStream_t s) {
+    constexpr size_t smem = pass_duo_smem<LOGR>();
+    auto kern = a.first ? k_fft_pass_duo<LOGR, true> : k_fft_pass_duo<LOGR, false>;
+    const cudaError_t e = raise_smem_limit((const void*)kern, smem);
+    if (e != cudaSuccess) return e;
+    const int64_t ntiles = (p->M >> PT_LOGE) * (int64_t)a.ng;
+    const unsigned blocks = (unsigned)std::min<int64_t>((ntiles + 1) / 2, device_sm_count());
+    kern<<<blocks, DUO_NT, smem, s>>>((const cpx<float>*)in, (cpx<float>*)out, a, p->d_L,
+                                      (const cpx<float>*)p->d_twlo, (const cpx<float>*)p->d_twhi,
+                                      (const cpx<float>*)p->d_twst + p->twst_off[LOGR], a.ng,
+                                      p->d_status,
+                                      p->dbg_wait_cycles > 0 ? p->dbg_wait_cycles : PT_WAIT_CYCLES,
+                                      p->dbg_drop_tile);
+    return cudaGetLastError();
+}
+
+template <int LOGR>
 static cudaError_t run_pass_tma(fc2_plan_s* p, const void* in, void* out, const PassArgs& a,
                                 cudaStream_t s) {
     constexpr int LOGJ = PT_LOGE - LOGR;
@@ -1914,7 +2233,10 @@ static cudaError_t run_radix(fc2_plan_s* p, const void* in, void* out, const Pas
         if (LOGR != p->logM && r32_pass(p->fft_family, LOGR)) return run_pass64<32, LOGR>(p, in, out, a, s);
     }
     if constexpr (sizeof(T) == 4 && LOGR >= 8 && LOGR <= 12) {
-        if (LOGR != p->logM && p->fft_family != FFT_R16) return run_pass_tma<LOGR>(p, in, out, a, s);
+        if (LOGR != p->logM && p->fft_family != FFT_R16) {
+            if constexpr (LOGR <= 9) return run_pass_duo<LOGR>(p, in, out, a, s);
+            else return run_pass_tma<LOGR>(p, in, out, a, s);
+        }
     }
     if (LOGR == p->logM) {
         constexpr int NT = (1 << LOGR) / 16 < 32 ? 32 : (1 << LOGR) / 16;
@@ -2103,6 +2425,20 @@ static int replay_plan(int logM, bool fp64, int family, const std::vector<int>& 
                         if (se < 0 || se >= E) return fail(pi, 6, bx, se);
                     }
                 }
+                continue;
+            }
+            if (sh.kind == PK_BULK && LOGR <= 9 && !first && logNs + LOGR + logRn == logM &&
+                logNs >= LOGJn && logNs >= LOGJ) {  // k_fft_pass_duo's direct middle store
+                for (int64_t kr = 0; kr < R; ++kr)
+                    for (int jj = 0; jj < J; ++jj) {
+                        const int64_t jl = (j0 + jj) & ((1ll << logNs) - 1), jh = (j0 + jj) >> logNs;
+                        const int64_t gi = (((jl >> LOGJn) + (kr << (logNs - LOGJn))) << logBlk) +
+                                           (jh << LOGJn) + (jl & ((1 << LOGJn) - 1));
+                        if (gi < 0 || gi >= M ||
+                            gi != blocked_pos(stockham_out(j0 + jj, (int)kr, logNs, LOGR), logSn, LOGJn,
+                                              logBlk))
+                            return fail(pi, 9, bx, gi);
+                    }
                 continue;
             }
             const bool rowcol = sh.kind == PK_R16 && same_radix;
