@@ -1754,6 +1754,116 @@ __global__ void __launch_bounds__(DUO_NT, 1) k_fft_pass_duo(const cpx<float>* __
     }
 }
 
+// ------------------------------------------- the 2^10 first pass
+// The first pass of radix 2^10 with the arithmetic of k_fft_pass64 (stage A
+// radix 16, stage B radix 64; results are bit-equal), by three groups of 128
+// threads per SM with an 8-column tile each: a thread holds 64 elements in 167
+// registers, and one group's loads, barriers and stores are covered by the other
+// two's arithmetic, where one group of 256 threads with one 16-column tile
+// waited for itself (issue active 47%).  Bound by the shared-memory and issue
+// rates together (without its stores it takes 9% less, without its loads 18%).
+// The tile has one slot of padding per two rows (16 columns of 8 bytes: all
+// banks): the column-wise and the row-wise accesses are free of conflicts, and
+// every access of an unrolled loop is a fixed offset from its thread's base.
+// Results leave along 16 rows of a column, one 128-byte line of the next
+// pass's layout per half-warp.
+//   1024 survey curves: 17.4 -> 13.6 ms (3.8 TB/s written); two groups 16.2;
+//   stage B split into 16-point transforms and merges for 16 warps of 32
+//   elements 16.7 (two more passes through shared memory); slots XORed with the
+//   row instead of padding 18.4 ms (addresses took 45% of the ALU pipe).
+constexpr int D10_LOGJ = 3;
+FC2_HD constexpr int d10_slot(int row, int jj) { return (row << D10_LOGJ) + (row >> 1) + jj; }
+constexpr int D10_TILE = d10_slot(1 << 10, 0);
+
+constexpr int D10_GT = 128, D10_NG = 3;   // threads of a group, groups
+constexpr size_t pass_d10_smem() { return (size_t)(D10_NG * D10_TILE + 63 * 16) * sizeof(cpx<float>); }
+FC2_D void d10_sync(int g) { asm volatile("bar.sync %0, 128;\n" ::"r"(g + 1) : "memory"); }
+__global__ void __launch_bounds__(D10_NG * D10_GT, 1) k_fft_first10(const cpx<float>* __restrict__ in,
+                                                        cpx<float>* __restrict__ out, PassArgs a,
+                                                        const int64_t* __restrict__ Lg,
+                                                        const cpx<float>* __restrict__ tw64, int G) {
+    using T = float;
+    constexpr int LOGR = 10, R = 1 << LOGR, QA = 16, J = 1 << D10_LOGJ;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int grp = threadIdx.x / D10_GT, gt = threadIdx.x % D10_GT;
+    cpx<T>* bufs = reinterpret_cast<cpx<T>*>(smem_raw);
+    cpx<T>* buf = bufs + grp * D10_TILE;
+    cpx<T>* st = bufs + D10_NG * D10_TILE;
+    const int M = 1 << a.logM, S = M >> LOGR;
+    const int tiles_x = S >> D10_LOGJ, ntiles = tiles_x * G;
+    for (int i = threadIdx.x; i < 63 * QA; i += D10_NG * D10_GT) st[i] = tw64[i];
+    __syncthreads();
+    auto rows_of = [&](int g) {
+        const int rows = (int)((Lg[g] + S - 1) / S);
+        return rows > R ? R : rows;
+    };
+    const int tstep = D10_NG * (int)gridDim.x;
+    // the next pass is the last one, of radix 2^9 in 16-column tiles (2^19 points)
+    const bool direct13 = a.logRn == 9 && a.logJn == 4 && a.logM == LOGR + 9;
+    for (int tile = blockIdx.x * D10_NG + grp; tile < ntiles; tile += tstep) {
+        const int gl = tile / tiles_x, g = a.g0 + gl, j0 = (tile - gl * tiles_x) * J;
+        const cpx<T>* gin = in + (int64_t)g * M;
+        const int rows = rows_of(g);
+        if (tile + tstep < ntiles) {  // ask L2 for the group's next tile
+            const int tn = tile + tstep, gnl = tn / tiles_x, gn = a.g0 + gnl;
+            const cpx<T>* ginn = in + (int64_t)gn * M + (tn - gnl * tiles_x) * J;
+            const int rn = rows_of(gn);
+            for (int r = gt; r < rn; r += D10_GT) prefetch_l2(ginn + (int64_t)r * S);
+        }
+        cpx<T> v[64];
+        // ---- stage A: radix 16, rows pp + 64 k -> rows 16 pp + k, pruned to the
+        // leading inputs that can be nonzero
+        auto stage_a = [&](auto mz_tag) {
+            constexpr int MZ = decltype(mz_tag)::value;
+#pragma unroll
+            for (int b = 0; b < 4; ++b) {
+                const int bi = gt + b * D10_GT, jj = bi & (J - 1), pp = bi >> D10_LOGJ;
+#pragma unroll
+                for (int k = 0; k < MZ; ++k) {
+                    const int r = pp + k * 64;
+                    v[b * 16 + k] = (r < rows) ? gin[j0 + jj + (int64_t)r * S] : mk<T>(0.f, 0.f);
+                }
+            }
+            d10_sync(grp);  // the previous tile's stage B has read the buffer
+#pragma unroll
+            for (int b = 0; b < 4; ++b) {
+                const int bi = gt + b * D10_GT, jj = bi & (J - 1), pp = bi >> D10_LOGJ;
+                if constexpr (MZ < QA) PrunedDFT<T, QA, MZ>::run(v + b * 16);
+                else SmallDFT<T, QA>::run(v + b * 16);
+#pragma unroll
+                for (int k = 0; k < 16; ++k) buf[d10_slot(pp * 16, jj) + d10_slot(k, 0)] = v[b * 16 + k];
+            }
+        };
+        const int kz = (rows + 63) >> 6;
+        if (kz <= 1) stage_a(std::integral_constant<int, 1>{});
+        else if (kz <= 2) stage_a(std::integral_constant<int, 2>{});
+        else if (kz <= 4) stage_a(std::integral_constant<int, 4>{});
+        else if (kz <= 8) stage_a(std::integral_constant<int, 8>{});
+        else stage_a(std::integral_constant<int, 16>{});
+        d10_sync(grp);
+        // ---- stage B: radix 64, lanes along 16 rows of a column
+        const int pp = gt & 15, jj = gt >> 4;
+        cpx<T>* gout = out + (int64_t)g * M;
+        cpx<T>* row0 = buf + d10_slot(pp, jj);
+#pragma unroll
+        for (int k = 0; k < 64; ++k) v[k] = row0[d10_slot(16 * k, 0)];
+#pragma unroll
+        for (int k = 1; k < 64; ++k) v[k] = mul(v[k], st[(k - 1) * QA + pp]);
+        SmallDFT<T, 64>::run(v);
+        if (direct13) {  // rows 16 k + pp: block k, row pp of it
+#pragma unroll
+            for (int k = 0; k < 64; ++k) gout[((j0 + jj) << 4) + pp + (k << 13)] = v[k];
+        } else {
+            d10_sync(grp);
+#pragma unroll
+            for (int k = 0; k < 64; ++k) row0[d10_slot(16 * k, 0)] = v[k];
+            d10_sync(grp);
+            store_tile_blocked<LOGR, D10_LOGJ, D10_GT>(
+                gout, buf, [](int e) { return d10_slot(e >> D10_LOGJ, e & (J - 1)); }, j0, a, gt);
+        }
+    }
+}
+
 // Whether a float pass of radix 2^logR runs on the radix-32 register kernel.
 static bool r32_pass(int family, int logR) {
     return (family == FFT_R32 && logR == 10) || (family == FFT_R32X && (logR == 9 || logR == 10));
@@ -2153,6 +2263,18 @@ static cudaError_t run_pass_d(fc2_plan_s* p, const void* in, void* out, const Pa
     return cudaGetLastError();
 }
 
+static cudaError_t run_first10(fc2_plan_s* p, const void* in, void* out, const PassArgs& a,
+                               cudaStream_t s) {
+    constexpr size_t smem = pass_d10_smem();
+    const cudaError_t e = raise_smem_limit((const void*)k_fft_first10, smem);
+    if (e != cudaSuccess) return e;
+    const int64_t ntiles = (p->M >> PT_LOGE) * (int64_t)a.ng;
+    const unsigned blocks = (unsigned)std::min<int64_t>((ntiles + D10_NG - 1) / D10_NG, device_sm_count());
+    k_fft_first10<<<blocks, D10_NG * D10_GT, smem, s>>>((const cpx<float>*)in, (cpx<float>*)out, a, p->d_L,
+                                               (const cpx<float>*)p->d_twst + p->tw64_off[10], a.ng);
+    return cudaGetLastError();
+}
+
 template <int RB, int LOGR>
 static cudaError_t run_pass64(fc2_plan_s* p, const void* in, void* out, const PassArgs& a,
                               cudaStream_t s) {
@@ -2227,7 +2349,10 @@ template <typename T, int LOGR>
 static cudaError_t run_radix(fc2_plan_s* p, const void* in, void* out, const PassArgs& a,
                              cudaStream_t s) {
     if constexpr (sizeof(T) == 4 && LOGR >= 10 && LOGR <= 12) {
-        if (LOGR != p->logM && p->fft_family == FFT_R64) return run_pass64<64, LOGR>(p, in, out, a, s);
+        if (LOGR != p->logM && p->fft_family == FFT_R64) {
+            if (LOGR == 10 && a.first) return run_first10(p, in, out, a, s);
+            return run_pass64<64, LOGR>(p, in, out, a, s);
+        }
     }
     if constexpr (sizeof(T) == 4 && (LOGR == 9 || LOGR == 10)) {
         if (LOGR != p->logM && r32_pass(p->fft_family, LOGR)) return run_pass64<32, LOGR>(p, in, out, a, s);
@@ -2337,7 +2462,10 @@ static int replay_plan(int logM, bool fp64, int family, const std::vector<int>& 
     for (int pi = 0; pi < P; ++pi) {
         const int LOGR = rs[pi];
         const int64_t R = 1ll << LOGR, S = M >> LOGR;
-        const PassShape sh = pass_shape(logM, fp64, family, LOGR);
+        PassShape sh = pass_shape(logM, fp64, family, LOGR);
+        // k_fft_first10: 8-column tiles, direct stores for two-pass plans
+        const bool first10 = sh.kind == PK_R64 && LOGR == 10 && pi == 0;
+        if (first10) sh = PassShape{PK_R64, PT_LOGE, D10_LOGJ, DUO_GT};
         const int LOGJ = sh.logj, J = 1 << LOGJ;
         const int64_t E = R << LOGJ;
         const bool first = pi == 0, last = pi == P - 1;

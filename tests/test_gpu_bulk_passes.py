@@ -1,4 +1,4 @@
-"""The 2^8 and 2^9 transform passes as first, middle and last passes, with grids
+"""The 2^8, 2^9 and (first) 2^10 transform passes as first, middle and last passes, with grids
 occupied in part (skipped zero levels) and throughout and trial grids of half
 the modes and fewer: spectra against the radix-16 family's."""
 import numpy as np
@@ -14,7 +14,9 @@ pytestmark = pytest.mark.gpu
     (1 << 15, 2, 0.03), (1 << 15, 2, 0.3), (25001, 2, 0.11), (1 << 14, 4, 0.3),
     (1 << 16, 2, 0.005), (1 << 16, 2, 0.45), (50021, 2, 0.2), (1 << 15, 4, 0.24),
     (1 << 17, 2, 0.06), (1 << 17, 2, 0.49), (100003, 2, 0.13), (1 << 16, 4, 0.3),
-    (1 << 24, 2, 0.2), (1 << 25, 2, 0.01)])
+    # 2^19 = 10 x 9 and 2^20 = 10 x 10: the 2^10 first pass, stored directly and staged
+    (1 << 18, 2, 0.03), (1 << 18, 2, 0.1), (1 << 18, 2, 0.45), (200003, 2, 0.25), (1 << 17, 4, 0.2),
+    (1 << 19, 2, 0.06), (400009, 2, 0.3), (1 << 24, 2, 0.2), (1 << 25, 2, 0.01)])
 def test_spectra_match_radix16_family(N, oversample, fill):
     from paper_0901_1913_gb300 import _fc2
     c = synth.short_curve(seed=5, n=300)
