@@ -518,8 +518,9 @@ static int64_t launches_front(const fc2_plan_s* p) {
     int64_t n = 1 + 1 + (int64_t)p->passes.size() + 1 + (p->fp64 ? 0 : 1);  // phase, spread, fft, assemble(+resolve)
     int bits = 0;
     while ((1ll << bits) < p->M + 2 * std::max(p->w, p->w_p) + 2) ++bits;
-    for (auto& g : p->geom)
-        if (g.wraps) n += 2 + 3 * ((bits + 7) / 8);
+    int64_t wraps = 0;
+    for (auto& g : p->geom) wraps += g.wraps ? 1 : 0;
+    if (wraps > 0) n += p->n <= RUN_CAP ? 1 : wraps * (2 + 3 * ((bits + 7) / 8));
     return n;
 }
 

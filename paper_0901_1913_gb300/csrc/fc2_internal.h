@@ -63,6 +63,10 @@ inline int fft_family_of(int fft_kernel) {
                              : FFT_R64;
 }
 
+// Longest sample set whose wrapping keys are ordered by its runs in one launch
+// (k_sort_runs); longer ones take the radix sort.
+constexpr int RUN_CAP = 7168;
+
 struct GridGeom {
     int k;            // harmonic multiple of this transform
     int kind;         // 0 = Q (weights), 1 = P (weighted data)
