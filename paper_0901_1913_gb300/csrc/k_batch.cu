@@ -200,6 +200,11 @@ constexpr double BX_EPS_DF = 1.5e-12;  // relative precision of the tier-2 (doub
 // relative pivot of the gridded equations below which an entry is taken as
 // nearly singular and starts at the double tier
 constexpr double BX_DMIN_T3 = 1e-7;
+// Smallest relative pivot used for routing.  Curves of fewer than 8 harmonics
+// count as nearly singular whatever their pivots (the empty columns of a system
+// padded to 8 do), so their flagged entries go straight to the last and most
+// precise tier, whichever capacity the solve is padded to.
+FC2_D double bx_pivot(double dmin, int H) { return H < 8 ? 0.0 : dmin; }
 
 // Double re-solve of listed (curve, bin) entries of the float path.  Entries
 // still too sensitive go on to the exact sums: to the float tier, straight to
@@ -224,7 +229,7 @@ __global__ void __launch_bounds__(128) k_bresolve(const cpx<float>* __restrict__
     int64_t cnt = *rcount;
     if (cnt > rcap) cnt = rcap;
     const int64_t wpb = blockDim.x >> 5;  // one entry per warp (warp-cooperative solve)
-    for (int64_t b = (int64_t)blockIdx.x * wpb + (threadIdx.x >> 5); b < cnt;
+    for (int64_t b = (int64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x; b < cnt;
          b += (int64_t)gridDim.x * wpb) {
         const int c = (int)(rlist[b] >> 32);
         const int64_t j = rlist[b] & 0xffffffffll;
@@ -254,7 +259,7 @@ __global__ void __launch_bounds__(128) k_bresolve(const cpx<float>* __restrict__
             S.pi[k] = (double)v.y * d * sp;
         }
         double o[HM], an2 = 0.0;
-        const double dmin = warp_chol_solve<HM, true>(S, tau, o, &an2, H);
+        const double dmin = bx_pivot(warp_chol_solve<HM, true>(S, tau, o, &an2, H), H);
         if ((threadIdx.x & 31) == 0) {
             const int m = 2 * H + 1;
             if (!(est_err<double>(an2, m, eps) <= err_fix)) {
@@ -517,7 +522,7 @@ __global__ void __launch_bounds__(BX_SPLIT_NT) k_bx_split(CurveTab ct,
 }
 
 // One warp per work item: the item's share of its entry's samples, summed
-// into row w of part (6 BHM doubles per row).
+// into row w of part (6 HM doubles per row).
 template <int HM, int TIER>
 __global__ void __launch_bounds__(BX_NT, TIER == 4 ? 2 : 1) k_bx_part(
     const uint64_t* __restrict__ Aph, const uint64_t* __restrict__ Bph,
@@ -531,7 +536,8 @@ __global__ void __launch_bounds__(BX_NT, TIER == 4 ? 2 : 1) k_bx_part(
     tb.load(dftab);
     const int nw = *nitems;
     const int lane = threadIdx.x & 31;
-    for (int w = blockIdx.x * BX_W + (threadIdx.x >> 5); w < nw; w += gridDim.x * BX_W) {
+    // items go to the CTAs in turn: few of them spread over all SMs
+    for (int w = (threadIdx.x >> 5) * gridDim.x + blockIdx.x; w < nw; w += gridDim.x * BX_W) {
         const int it = items[w];
         const int64_t e = it / BX_QMAX;
         const int q = it % BX_QMAX;
@@ -569,7 +575,7 @@ __global__ void __launch_bounds__(BX_NT) k_bexact(
     int64_t cnt = *count;
     if (cnt > cap) cnt = cap;
     const int lane = threadIdx.x & 31;
-    for (int64_t e = (int64_t)blockIdx.x * BX_W + (threadIdx.x >> 5); e < cnt;
+    for (int64_t e = (int64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x; e < cnt;
          e += (int64_t)gridDim.x * BX_W) {
         const int64_t ent = list[e];
         const int c = (int)(ent >> 32);
@@ -592,7 +598,7 @@ __global__ void __launch_bounds__(BX_NT) k_bexact(
             double lo = 0.0, hi = 0.0;
             for (int q = 0; q < nq; ++q) {
                 const double* row = part + (int64_t)(qb + q) * NV;
-                lo += row[lane];
+                if (lane < NV) lo += row[lane];
                 if (lane + 32 < NV) hi += row[lane + 32];
             }
 #pragma unroll
@@ -608,7 +614,7 @@ __global__ void __launch_bounds__(BX_NT) k_bexact(
         const double chi0 = sc[SC_CHI0];
         if constexpr (MODE == 0) {
             double o[HM], an2 = 0.0;
-            const double dmin = warp_chol_solve<HM, true>(S, tau_drop, o, &an2, H);
+            const double dmin = bx_pivot(warp_chol_solve<HM, true>(S, tau_drop, o, &an2, H), H);
             const double eps = TIER == 1 ? 2e-7 * sc[SC_RW] : (TIER == 2 ? BX_EPS_DF : 1e-14);
             // sums cannot vouch for a pivot near their precision (their errors
             // can also make the coefficients look small): such entries go on
@@ -1040,6 +1046,7 @@ struct Batch {
     double tune_ms = 0;
     int tune_timed = 0;
     int64_t launches = 0;
+    int hmax = 8;              // most harmonics of the call's curves
     int64_t stats[4] = {0, 0, 0, 0};
     double phase_ms[7] = {0, 0, 0, 0, 0, 0, 0};  // host wall time of the call's phases
     // stage timing (fc2_debug_batch_timing): events recorded on the stream between
@@ -1216,64 +1223,77 @@ static cudaError_t chunk_launches(Batch& b, int nc, int64_t ntot, int64_t nmax, 
 #undef FC2_BASM
         ++nl;
     }
-    if (f32) {
-        k_bresolve<BHM><<<4 * 152, 128, 0, s>>>((const cpx<float>*)p.d_spec, (const float*)p.d_dec,
-                                                N, ct, tau_drop, eps_spec, err_fix, out, b.list,
-                                                b.counts + 0, (int64_t)b.cl1, b.list2, b.counts + 1,
-                                                (int64_t)b.cl2, b.list3, b.counts + 2,
-                                                (int64_t)b.cl3, b.list4, b.counts + 3,
-                                                (int64_t)b.cl4);
-        ++nl;
-    }
-    mark(3);
-    // exact fix-up: float sums over list2 (escalating to list3), double-float
-    // sums over list3 (escalating to list4), double sums over list4
-    const dfc* tab = (const dfc*)b.dftab;
-    const unsigned gx = 2 * 152;
-    int32_t* nitems = b.counts + 10;
-    // one tier (or the records) over `list`: number the work items, sum them,
-    // then add, solve and route each entry
-    auto exact = [&](auto tier_tag, auto mode_tag, const int64_t* list, const int32_t* cnt,
-                     int64_t cap, double tau, int64_t* next, int32_t* next_cnt, int64_t next_cap,
-                     fc2_best* recs) {
-        constexpr int TIER = decltype(tier_tag)::value, MODE = decltype(mode_tag)::value;
-        k_bx_split<<<1, BX_SPLIT_NT, 0, s>>>(ct, list, cnt, cap, b.qbase, b.items, nitems);
-        k_bx_part<BHM, TIER><<<gx, BX_NT, 0, s>>>(b.A, b.B, b.wq32, b.wp32, b.wq, b.wp, tab, ntot,
-                                                  ct, list, b.items, nitems, b.part);
-        k_bexact<BHM, TIER, MODE><<<gx, BX_NT, 0, s>>>(b.A, b.B, b.wq32, b.wp32, b.wq, b.wp, tab,
-                                                       ntot, ct, N, list, cnt, cap, b.qbase, b.part,
-                                                       tau, err_fix, out, next, next_cnt, next_cap,
-                                                       recs);
-        nl += 3;
+    // Re-solve, exact sums and records: their systems are padded to a harmonic
+    // capacity of 4, 6 or 8, the smallest that holds the call's curves (one
+    // capacity for every chunk, so that the chunks' graphs have one shape).  A
+    // warp's double solve of the 17-square padded system takes three times the
+    // double instructions of the 9-square one: 512 curves of four harmonics
+    // spent 1.53 ms in the solves at capacity 8, 0.75 at 4; 1024 curves of 2..6 3.2
+    // ms at 8, 2.2 at 6.
+    auto tail = [&](auto hm_tag) {
+        constexpr int HM = decltype(hm_tag)::value;
+        if (f32) {
+            k_bresolve<HM><<<4 * 152, 128, 0, s>>>((const cpx<float>*)p.d_spec, (const float*)p.d_dec,
+                                                    N, ct, tau_drop, eps_spec, err_fix, out, b.list,
+                                                    b.counts + 0, (int64_t)b.cl1, b.list2, b.counts + 1,
+                                                    (int64_t)b.cl2, b.list3, b.counts + 2,
+                                                    (int64_t)b.cl3, b.list4, b.counts + 3,
+                                                    (int64_t)b.cl4);
+            ++nl;
+        }
+        mark(3);
+        // exact fix-up: float sums over list2 (escalating to list3), double-float
+        // sums over list3 (escalating to list4), double sums over list4
+        const dfc* tab = (const dfc*)b.dftab;
+        const unsigned gx = 2 * 152;
+        int32_t* nitems = b.counts + 10;
+        // one tier (or the records) over `list`: number the work items, sum them,
+        // then add, solve and route each entry
+        auto exact = [&](auto tier_tag, auto mode_tag, const int64_t* list, const int32_t* cnt,
+                         int64_t cap, double tau, int64_t* next, int32_t* next_cnt, int64_t next_cap,
+                         fc2_best* recs) {
+            constexpr int TIER = decltype(tier_tag)::value, MODE = decltype(mode_tag)::value;
+            k_bx_split<<<1, BX_SPLIT_NT, 0, s>>>(ct, list, cnt, cap, b.qbase, b.items, nitems);
+            k_bx_part<HM, TIER><<<gx, BX_NT, 0, s>>>(b.A, b.B, b.wq32, b.wp32, b.wq, b.wp, tab, ntot,
+                                                      ct, list, b.items, nitems, b.part);
+            k_bexact<HM, TIER, MODE><<<gx, BX_NT, 0, s>>>(b.A, b.B, b.wq32, b.wp32, b.wq, b.wp, tab,
+                                                           ntot, ct, N, list, cnt, cap, b.qbase, b.part,
+                                                           tau, err_fix, out, next, next_cnt, next_cap,
+                                                           recs);
+            nl += 3;
+        };
+        using I0 = std::integral_constant<int, 0>;
+        using I1 = std::integral_constant<int, 1>;
+        using I2 = std::integral_constant<int, 2>;
+        using I3 = std::integral_constant<int, 3>;
+        using I4 = std::integral_constant<int, 4>;
+        exact(I1{}, I0{}, b.list2, b.counts + 1, (int64_t)b.cl2, 1e-13, b.list3, b.counts + 2,
+              (int64_t)b.cl3, nullptr);
+        exact(I2{}, I0{}, b.list3, b.counts + 2, (int64_t)b.cl3, 1e-13, b.list4, b.counts + 3,
+              (int64_t)b.cl4, nullptr);
+        // the last tier: sums exact in fixed point on the float and integer pipes for
+        // the mixed path, double sums for the FP64 path
+        if (f32 && !b.double_last)
+            exact(I4{}, I0{}, b.list4, b.counts + 3, (int64_t)b.cl4, 1e-13, nullptr, nullptr, 0,
+                  nullptr);
+        else
+            exact(I3{}, I0{}, b.list4, b.counts + 3, (int64_t)b.cl4, 1e-13, nullptr, nullptr, 0,
+                  nullptr);
+        mark(4);
+        if (K > 0) {
+            const int nblk = (int)((N + BP_B - 1) / BP_B);
+            k_bpeaks0<<<dim3((unsigned)nblk, (unsigned)nc), BP_NT, 0, s>>>(out, N, ct, nblk, b.bbest);
+            k_bpeaks_theta<<<(unsigned)nc, 256, 0, s>>>(b.bbest, nblk, K, b.theta);
+            k_bpeaks1<<<dim3((unsigned)nblk, (unsigned)nc), BP_NT, 0, s>>>(out, N, ct, K, nblk, b.bbest,
+                                                                            b.theta, b.tops);
+            k_bpeaks2<<<(unsigned)nc, 256, 0, s>>>(b.tops, nblk, K, b.pent);
+            nl += 4;
+            exact(I2{}, I1{}, b.pent, b.counts + 4, nrec, tau_drop, nullptr, nullptr, 0, b.recs_now);
+        }
     };
-    using I0 = std::integral_constant<int, 0>;
-    using I1 = std::integral_constant<int, 1>;
-    using I2 = std::integral_constant<int, 2>;
-    using I3 = std::integral_constant<int, 3>;
-    using I4 = std::integral_constant<int, 4>;
-    exact(I1{}, I0{}, b.list2, b.counts + 1, (int64_t)b.cl2, 1e-13, b.list3, b.counts + 2,
-          (int64_t)b.cl3, nullptr);
-    exact(I2{}, I0{}, b.list3, b.counts + 2, (int64_t)b.cl3, 1e-13, b.list4, b.counts + 3,
-          (int64_t)b.cl4, nullptr);
-    // the last tier: sums exact in fixed point on the float and integer pipes for
-    // the mixed path, double sums for the FP64 path
-    if (f32 && !b.double_last)
-        exact(I4{}, I0{}, b.list4, b.counts + 3, (int64_t)b.cl4, 1e-13, nullptr, nullptr, 0,
-              nullptr);
-    else
-        exact(I3{}, I0{}, b.list4, b.counts + 3, (int64_t)b.cl4, 1e-13, nullptr, nullptr, 0,
-              nullptr);
-    mark(4);
-    if (K > 0) {
-        const int nblk = (int)((N + BP_B - 1) / BP_B);
-        k_bpeaks0<<<dim3((unsigned)nblk, (unsigned)nc), BP_NT, 0, s>>>(out, N, ct, nblk, b.bbest);
-        k_bpeaks_theta<<<(unsigned)nc, 256, 0, s>>>(b.bbest, nblk, K, b.theta);
-        k_bpeaks1<<<dim3((unsigned)nblk, (unsigned)nc), BP_NT, 0, s>>>(out, N, ct, K, nblk, b.bbest,
-                                                                        b.theta, b.tops);
-        k_bpeaks2<<<(unsigned)nc, 256, 0, s>>>(b.tops, nblk, K, b.pent);
-        nl += 4;
-        exact(I2{}, I1{}, b.pent, b.counts + 4, nrec, tau_drop, nullptr, nullptr, 0, b.recs_now);
-    }
+    if (b.hmax <= 4) tail(std::integral_constant<int, 4>{});
+    else if (b.hmax <= 6) tail(std::integral_constant<int, 6>{});
+    else tail(std::integral_constant<int, BHM>{});
     mark(5);
     b.launches += nl;
     return cudaGetLastError();
@@ -1653,6 +1673,7 @@ fc2_status batched_execute(int64_t C, const int64_t* offsets, const double* t, c
         }
     }
     Batch b;
+    b.hmax = *std::max_element(Hc, Hc + C);
     if (opt.cuda_stream) b.s = (cudaStream_t)opt.cuda_stream;
     else {
         if (cudaStreamCreateWithFlags(&b.s, cudaStreamNonBlocking) != cudaSuccess) return FC2_ERR_CUDA;
