@@ -45,12 +45,21 @@ struct Sys {
 FC2_D float inv_sqrt(float d) { return rsqrtf(d); }
 FC2_D double inv_sqrt(double d) { return 1.0 / sqrt(d); }
 
+// A value for the error estimate in float; doubles are narrowed on the integer
+// pipes (truncating; magnitudes outside the float range give 0 or infinity).
+FC2_D float narrow_est(float v) { return v; }
+FC2_D float narrow_est(double v) {
+    return copysignf(d2f_trunc(fabs(v)), (float)(__double2hiint(v) >> 31 | 1));
+}
+
 // Factor and solve; out[H'-1] = Delta chi^2'_{H'}.  Returns the minimum
 // relative pivot over all columns (clamped at 0).  With COEF, *anorm2 receives
 // max over H' of |A^{(H')}|^2 (A^{(H')} = the H'-harmonic coefficients, by
 // back-substitution L^T A = z on the leading block), the sensitivity of the
-// result to errors in alpha and beta.  Optionally keeps L and z.
-template <typename TC, int H, bool COEF>
+// result to errors in alpha and beta.  Optionally keeps L and z.  RSQRT: double
+// reciprocal roots by rsqrt (some 13 double operations less each; its last bit
+// differs), where the result is returned in float.
+template <typename TC, int H, bool COEF, bool RSQRT = false>
 FC2_D TC chol_solve(const Sys<TC, H>& S, TC tau, TC* out, TC* anorm2,
                     TC (*Lkeep)[2 * H + 1] = nullptr, TC* zkeep = nullptr, int Hrun = H) {
     constexpr int m = 2 * H + 1;
@@ -77,7 +86,9 @@ FC2_D TC chol_solve(const Sys<TC, H>& S, TC tau, TC* out, TC* anorm2,
         // quotient itself only feeds the returned minimum (and is dropped by
         // the compiler when a caller ignores it)
         if (all > (TC)0 && d > tau * all) {
-            const TC di = inv_sqrt(d);
+            TC di;
+            if constexpr (RSQRT) di = rsqrt(d);
+            else di = inv_sqrt(d);
             L[l][l] = d * di;
             dinv[l] = di;
             z[l] = b * di;
@@ -93,27 +104,36 @@ FC2_D TC chol_solve(const Sys<TC, H>& S, TC tau, TC* out, TC* anorm2,
         if (l > 0 && (l & 1) == 0) out[(l >> 1) - 1] = acc;
     }
     if constexpr (COEF) {
-        TC amax = (TC)0;
+        // in float also for a double solve: the norm only feeds the error estimate,
+        // and its back-substitutions were 20-25% of the double operations
+        // (32 curves, N = 2^18, H = 2..6: 9.4 -> 8.3 ms; 2^20 bins, H = 4: 1086 -> 965 us)
+        float Lf[m][m], zf[m], df[m], amax = 0.f;
+#pragma unroll
+        for (int l = 0; l < m; ++l) {
+            zf[l] = narrow_est(z[l]);
+            df[l] = narrow_est(dinv[l]);
+#pragma unroll
+            for (int k = 0; k < l; ++k) Lf[l][k] = narrow_est(L[l][k]);
+        }
 #pragma unroll
         for (int hp = 1; hp <= H; ++hp) {
             if (hp > Hrun) break;  // harmonics beyond the curve's own H are padding
             const int mp = 2 * hp + 1;
-            TC A[m];
-            TC nrm = (TC)0;
+            float A[m], nrm = 0.f;
 #pragma unroll
             for (int l = m - 1; l >= 0; --l) {
                 if (l < mp) {
-                    TC a = z[l];
+                    float a = zf[l];
 #pragma unroll
                     for (int k = l + 1; k < m; ++k)
-                        if (k < mp) a = fma(-L[k][l], A[k], a);
-                    A[l] = a * dinv[l];
-                    nrm = fma(A[l], A[l], nrm);
+                        if (k < mp) a = fmaf(-Lf[k][l], A[k], a);
+                    A[l] = a * df[l];
+                    nrm = fmaf(A[l], A[l], nrm);
                 }
             }
             amax = nrm > amax ? nrm : amax;
         }
-        *anorm2 = amax;
+        *anorm2 = (TC)amax;
     }
     if (Lkeep) {
 #pragma unroll

@@ -185,7 +185,7 @@ __global__ void __launch_bounds__(NT) k_bassemble(const cpx<TS>* __restrict__ sp
         S.pi[k] = v.y * dp;
     }
     TS o[H], an2 = (TS)0;
-    chol_solve<TS, H, true>(S, tau, o, &an2);
+    chol_solve<TS, H, true, sizeof(TS) == 8>(S, tau, o, &an2);
     if (!(est_err<TS>(an2, 2 * H + 1, eps) <= err_fix)) {
         const int32_t pos = atomicAdd(list_count, 1);
         if (pos < cap) list[pos] = ((int64_t)c << 32) | j;

@@ -174,9 +174,6 @@ FC2_D void warp_joint_solve(const Sys<double, H>& S, const double* Tre, const do
 // spectra: 6036 -> 313 us (double pipe alone: about 220 us).
 FC2_D double widen(float v) { return f2d_exact(v); }
 FC2_D double widen(double v) { return v; }
-// double -> float for the error estimate, on the integer pipes (truncating;
-// magnitudes outside the float range give 0 or infinity).
-FC2_D float narrow_est(double v) { return copysignf(d2f_trunc(fabs(v)), (float)(__double2hiint(v) >> 31 | 1)); }
 
 template <typename TS, int H, int D>
 __global__ void __launch_bounds__(128) k_assemble_joint(const cpx<TS>* __restrict__ spec,
