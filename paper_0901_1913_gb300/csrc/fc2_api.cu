@@ -123,6 +123,7 @@ void free_plan_memory(fc2_plan_s* p) {
     dfree(p->d_key, s); dfree(p->d_dlt, s); dfree(p->d_cs, s);
     dfree(p->d_grid[0], s); dfree(p->d_grid[1], s); dfree(p->d_spec, s);
     dfree(p->d_dec, s); dfree(p->d_dec_p, s); dfree(p->d_twlo, s); dfree(p->d_twhi, s); dfree(p->d_twst, s);
+    dfree(p->d_twpass, s);
     dfree(p->d_dchi2, s); dfree(p->d_flag_list, s); dfree(p->d_flag_count, s);
     dfree(p->d_L, s); dfree(p->d_red, s); dfree(p->d_best, s); dfree(p->d_part, s);
     dfree(p->d_phA, s); dfree(p->d_phB, s); dfree(p->d_wq32, s); dfree(p->d_wp32, s);
@@ -244,8 +245,12 @@ fc2_status fc2_plan_create(const double* t, const double* x, const double* sigma
     const int NSRC = p->nsrc ? p->nsrc : G;  // sample sets
     const size_t spec_rows = p->packed ? (size_t)2 * G : (size_t)G;
     const size_t spec_bytes = p->paper ? (size_t)M * csz : spec_rows * N * csz;
+    // with the autotuner the passes may change: room for any plan's tables (each
+    // pass after the first needs at most the grid length, or one tile)
+    const int64_t tw_pass = !p->fp64 ? 0 : (opt.autotune > 0 ? 4 * std::max<int64_t>(M, 4096)
+                                                             : plan_pass_tw_entries(p));
     // memory estimate
-    size_t need = 0;
+    size_t need = (size_t)tw_pass * csz;
     need += (size_t)n * 8 * 6 + (size_t)n * 4;
     need += (size_t)NSRC * n * (4 + tsz + csz);
     need += 2 * (size_t)G * M * csz;
@@ -298,6 +303,7 @@ fc2_status fc2_plan_create(const double* t, const double* x, const double* sigma
         g.ok(dalloc(&p->d_best, (size_t)(H + p->top_k) * sizeof(fc2_best), s));
     p->flag_cap = N;
     p->exact_cap = std::max<int64_t>(2048, H + p->top_k);
+    if (tw_pass > 0) g.ok(dalloc(&p->d_twpass, (size_t)tw_pass * csz, s));
     if (p->joint) g.ok(dalloc(&p->d_part_t, trend_part_bytes(p->exact_cap, H, p->D), s));
     g.ok(dalloc(&p->d_part, exact_scratch_bytes(n, H, p->exact_cap), s)) &&
         g.ok(dalloc(&p->d_phA, (size_t)n * 8, s)) && g.ok(dalloc(&p->d_phB, (size_t)n * 8, s)) &&

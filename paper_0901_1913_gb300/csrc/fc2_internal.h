@@ -146,6 +146,7 @@ struct fc2_plan_s {
     void* d_twhi = nullptr;
     int tw_shift = 0;
     void* d_twst = nullptr;    // cpx<T> in-CTA stage twiddles per radix
+    void* d_twpass = nullptr;  // double plans: inter-pass twiddles in tile order
     int64_t twst_off[16] = {0};
     int64_t tw64_off[16] = {0};
     int fft_family = fc2::FFT_R64;  // kernel family of the float passes (fc2::FftFamily)
@@ -242,6 +243,7 @@ cudaError_t launch_detrend(const double* t, const double* x, const double* sigma
 
 // k_fft.cu
 void twiddle_split(int logM, bool fused, int* sh, int64_t* nlo, int64_t* nhi);  // d_twlo, d_twhi entries
+int64_t plan_pass_tw_entries(const fc2_plan_s* p);  // d_twpass entries (0: none)
 cudaError_t init_twiddles(fc2_plan_s* p, cudaStream_t s);
 cudaError_t init_deconv(fc2_plan_s* p, cudaStream_t s);
 void plan_fft_passes(fc2_plan_s* p);

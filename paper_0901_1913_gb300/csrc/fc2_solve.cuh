@@ -58,7 +58,8 @@ FC2_D float narrow_est(double v) {
 // back-substitution L^T A = z on the leading block), the sensitivity of the
 // result to errors in alpha and beta.  Optionally keeps L and z.  RSQRT: double
 // reciprocal roots by rsqrt (some 13 double operations less each; its last bit
-// differs), where the result is returned in float.
+// differs), where the result is returned in float (32 curves, N = 2^18, H = 2..6:
+// 8.3 -> 7.5 ms).
 template <typename TC, int H, bool COEF, bool RSQRT = false>
 FC2_D TC chol_solve(const Sys<TC, H>& S, TC tau, TC* out, TC* anorm2,
                     TC (*Lkeep)[2 * H + 1] = nullptr, TC* zkeep = nullptr, int Hrun = H) {

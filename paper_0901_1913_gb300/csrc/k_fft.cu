@@ -579,6 +579,63 @@ FC2_D void store_tile_blocked(cpx<T>* __restrict__ gout, const cpx<T>* s, SIdx s
     }
 }
 
+// SmallDFT<T, Q> of v when only v[0..MZ) can be nonzero: the same operations
+// without those on the zeros.
+template <typename T, int Q, int MZ>
+struct ZeroDFT {
+    static FC2_D void run(cpx<T>* v) {
+        if constexpr (MZ == Q) {
+            SmallDFT<T, Q>::run(v);
+        } else if constexpr (MZ == 1) {
+#pragma unroll
+            for (int k = 1; k < Q; ++k) v[k] = v[0];
+        } else {
+            cpx<T> e[Q / 2], o[Q / 2];
+#pragma unroll
+            for (int i = 0; i < MZ / 2; ++i) { e[i] = v[2 * i]; o[i] = v[2 * i + 1]; }
+            ZeroDFT<T, Q / 2, MZ / 2>::run(e);
+            ZeroDFT<T, Q / 2, MZ / 2>::run(o);
+#pragma unroll
+            for (int k = 0; k < Q / 2; ++k) {
+                cpx<T> t;
+                if (k == 0) t = o[k];
+                else if (4 * k == Q) t = mul_i(o[k]);
+                else if constexpr (Q <= 16) t = mul(o[k], root16<T>(k * (16 / Q)));
+                else t = mul(o[k], root64<T>(k * (64 / Q)));
+                v[k] = add(e[k], t);
+                v[k + Q / 2] = sub(e[k], t);
+            }
+        }
+    }
+};
+
+// The 16-point transform of SmallDFT<T, 16> where only outputs 0..3 and
+// 12..15 are wanted (a last pass that keeps the centred half of the modes):
+// the same operations for those outputs, the other eight not formed.
+template <typename T>
+FC2_D void dft16_centred(cpx<T>* v) {
+    cpx<T> e[8], o[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) { e[i] = v[2 * i]; o[i] = v[2 * i + 1]; }
+    SmallDFT<T, 8>::run(e);
+    SmallDFT<T, 8>::run(o);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) v[k] = add(e[k], k == 0 ? o[0] : mul(o[k], root16<T>(k)));
+#pragma unroll
+    for (int k = 4; k < 8; ++k) v[k + 8] = sub(e[k], k == 4 ? mul_i(o[4]) : mul(o[k], root16<T>(k)));
+}
+
+// Offset of the twiddles of the stage that follows 2^DONE (k_init_stage_tw).
+FC2_HD constexpr int stage_tw_offset(int LOGR, int DONE) {
+    int off = 0, done = 0;
+    while (done < DONE) {
+        const int qb = stage_bits(LOGR, done);
+        if (done > 0) off += ((1 << qb) - 1) * (1 << done);
+        done += qb;
+    }
+    return off;
+}
+
 // ------------------------------------------------------- double-precision pass
 // Bound by the double pipe (a warp's double instruction takes 64 clocks of its
 // sub-partition), so what counts is the double operations per element:
@@ -668,12 +725,54 @@ FC2_D void dit_stage(cpx<double>* v, int idx, int logP, const Tw& tw) {
     for (int i = 0; i < Q; ++i) v[i] = x[i];
 }
 
-// The pass of k_fft_pass in double: the same tiles, layouts and stages.
-template <int LOGR, int LOGJ, int NT>
+// The inter-pass twiddles of a pass after passes of radix product 2^logD in the
+// order its tiles hold their elements (they repeat with period 2^logD in the
+// columns): base step^k of each first-stage butterfly, formed as cta_stage
+// forms it, so a product with a table entry has cta_stage's bits.
+FC2_HD int64_t pass_tw_tiles(int logD, int LOGJ) { return logD > LOGJ ? 1ll << (logD - LOGJ) : 1; }
+template <int LOGR, int LOGJ>
+__global__ void k_init_pass_tw(cpx<double>* __restrict__ tab, int logM, int logD,
+                               const cpx<double>* __restrict__ twlo,
+                               const cpx<double>* __restrict__ twhi, int tws) {
+    using T = double;
+    constexpr int R = 1 << LOGR, J = 1 << LOGJ, Q = 1 << stage_bits(LOGR, 0);
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= pass_tw_tiles(logD, LOGJ) * (R / Q) * J) return;
+    const int64_t tile = i / ((R / Q) * J);
+    const int bi = (int)(i - tile * ((R / Q) * J)), jj = bi % J, pp = bi / J;
+    const int jm = (int)((tile * J + jj) & ((1 << logD) - 1)), lts = logM - logD - LOGR;
+    const cpx<T> base = twiddle(twlo, twhi, tws, (int64_t)((pp * jm) << lts));
+    const cpx<T> st1 = twiddle(twlo, twhi, tws, (int64_t)(((R / Q) * jm) << lts));
+    cpx<T> lo[4], hi[4];
+    lo[1] = st1;
+    lo[2] = mul(st1, st1);
+    lo[3] = mul(lo[2], st1);
+    hi[1] = mul(lo[2], lo[2]);
+    hi[2] = mul(hi[1], hi[1]);
+    hi[3] = mul(hi[2], hi[1]);
+    cpx<T>* t = tab + tile * R * J;
+#pragma unroll
+    for (int k = 0; k < Q; ++k) {
+        cpx<T> w = base;
+        if ((k & 3) != 0) w = mul(w, lo[k & 3]);
+        if ((k >> 2) != 0) w = mul(w, hi[k >> 2]);
+        t[(pp + k * (R / Q)) * J + jj] = w;
+    }
+}
+
+// The pass of k_fft_pass in double: the same tiles, layouts and stages.  FUSED
+// (batches): dit_stage's butterflies with the merged twiddles of the table twf
+// (q < M / 2).  Otherwise (plans) k_fft_pass's operations in its order, results
+// bit-equal, with the inter-pass twiddles from a table (twf, k_init_pass_tw: four
+// operations per element where forming them took eleven) and the zero rows and
+// unwanted modes skipped (12 grids of 2^21: 3.71 -> 3.11 ms); twst: the stage
+// twiddles.
+template <int LOGR, int LOGJ, int NT, bool FUSED>
 __global__ void __launch_bounds__(NT, 2) k_fft_pass_d(const cpx<double>* __restrict__ in,
                                                       cpx<double>* __restrict__ out, PassArgs a,
                                                       const int64_t* __restrict__ Lg,
-                                                      const cpx<double>* __restrict__ twf) {
+                                                      const cpx<double>* __restrict__ twf,
+                                                      const cpx<double>* __restrict__ twst) {
     constexpr int R = 1 << LOGR, J = 1 << LOGJ, E = R * J;
     constexpr int QB1 = stage_bits(LOGR, 0), QB2 = 4, NST = 1 + (LOGR - QB1) / 4;
     static_assert(QB1 + 4 * (NST - 1) == LOGR && NST >= 2 && NST <= 3, "two or three stages");
@@ -714,8 +813,23 @@ __global__ void __launch_bounds__(NT, 2) k_fft_pass_d(const cpx<double>* __restr
             const int bi = threadIdx.x + b * NT, jj = bi % J, pp = bi / J;
 #pragma unroll
             for (int k = 0; k < MZ; ++k) v[b][k] = s[phys((pp + k * (R / Q)) * J + jj)];
-            const int idx = ((j0 + jj) & maskD) + ((pp & (NS - 1)) << logD);
-            dit_stage<QB, MZ, decltype(tw_tag)::value, decltype(cen_tag)::value>(v[b], idx, logP, twc);
+            if constexpr (FUSED) {
+                const int idx = ((j0 + jj) & maskD) + ((pp & (NS - 1)) << logD);
+                dit_stage<QB, MZ, decltype(tw_tag)::value, decltype(cen_tag)::value>(v[b], idx, logP, twc);
+            } else {
+                constexpr int TOFF = stage_tw_offset(LOGR, DONE);
+                if constexpr (DONE == 0 && decltype(tw_tag)::value) {
+                    const cpx<double>* wt = twf + ((int64_t)(blockIdx.x & (pass_tw_tiles(logD, LOGJ) - 1))) * E;
+#pragma unroll
+                    for (int k = 0; k < Q; ++k) v[b][k] = mul(v[b][k], wt[(pp + k * (R / Q)) * J + jj]);
+                } else if constexpr (DONE > 0) {
+#pragma unroll
+                    for (int k = 1; k < MZ; ++k)
+                        v[b][k] = mul(v[b][k], twst[TOFF + (k - 1) * NS + (pp & (NS - 1))]);
+                }
+                if constexpr (decltype(cen_tag)::value) dft16_centred(v[b]);
+                else ZeroDFT<double, Q, MZ>::run(v[b]);
+            }
         }
         put(v);
     };
@@ -1160,22 +1274,6 @@ FC2_D bool mbar_wait_bounded(uint64_t* m, unsigned parity, long long cycles) {
     return true;
 }
 
-// The 16-point transform of SmallDFT<T, 16> where only outputs 0..3 and
-// 12..15 are wanted (a last pass that keeps the centred half of the modes):
-// the same operations for those outputs, the other eight not formed.
-template <typename T>
-FC2_D void dft16_centred(cpx<T>* v) {
-    cpx<T> e[8], o[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) { e[i] = v[2 * i]; o[i] = v[2 * i + 1]; }
-    SmallDFT<T, 8>::run(e);
-    SmallDFT<T, 8>::run(o);
-#pragma unroll
-    for (int k = 0; k < 4; ++k) v[k] = add(e[k], k == 0 ? o[0] : mul(o[k], root16<T>(k)));
-#pragma unroll
-    for (int k = 4; k < 8; ++k) v[k + 8] = sub(e[k], k == 4 ? mul_i(o[4]) : mul(o[k], root16<T>(k)));
-}
-
 // First-stage radix bits of the bulk-copy passes: radix 32 for 2^9 (two stages,
 // 32 x 16), else as the other shared-memory stages (2^9 would otherwise take
 // 2 x 16 x 16, one more pass through shared memory).
@@ -1463,36 +1561,6 @@ FC2_D bool duo_sync_and(int g, bool ok) {
         : "memory");
     return r != 0;
 }
-
-// SmallDFT<T, Q> of v when only v[0..MZ) can be nonzero: the same operations
-// without those on the zeros.
-template <typename T, int Q, int MZ>
-struct ZeroDFT {
-    static FC2_D void run(cpx<T>* v) {
-        if constexpr (MZ == Q) {
-            SmallDFT<T, Q>::run(v);
-        } else if constexpr (MZ == 1) {
-#pragma unroll
-            for (int k = 1; k < Q; ++k) v[k] = v[0];
-        } else {
-            cpx<T> e[Q / 2], o[Q / 2];
-#pragma unroll
-            for (int i = 0; i < MZ / 2; ++i) { e[i] = v[2 * i]; o[i] = v[2 * i + 1]; }
-            ZeroDFT<T, Q / 2, MZ / 2>::run(e);
-            ZeroDFT<T, Q / 2, MZ / 2>::run(o);
-#pragma unroll
-            for (int k = 0; k < Q / 2; ++k) {
-                cpx<T> t;
-                if (k == 0) t = o[k];
-                else if (4 * k == Q) t = mul_i(o[k]);
-                else if constexpr (Q <= 16) t = mul(o[k], root16<T>(k * (16 / Q)));
-                else t = mul(o[k], root64<T>(k * (64 / Q)));
-                v[k] = add(e[k], t);
-                v[k + Q / 2] = sub(e[k], t);
-            }
-        }
-    }
-};
 
 template <int LOGR>
 constexpr size_t pass_duo_smem() {
@@ -1889,6 +1957,28 @@ void twiddle_split(int logM, bool fused, int* sh, int64_t* nlo, int64_t* nhi) {
     *nhi = (1ll << logM) >> *sh;
 }
 
+// Entries of the inter-pass twiddle table of a double pass (0 for a first pass).
+static int64_t pass_tw_entries(int logM, int logR, int64_t Ns) {
+    if (Ns <= 1 || logR >= logM) return 0;
+    int logD = 0;
+    while ((1ll << logD) < Ns) ++logD;
+    return pass_tw_tiles(logD, FftCfg<double>::LOGE - logR) << FftCfg<double>::LOGE;
+}
+int64_t plan_pass_tw_entries(const fc2_plan_s* p) {
+    int64_t n = 0;
+    if (p->fp64 && !p->fused_fft)
+        for (const auto& ps : p->passes) n += pass_tw_entries(p->logM, ps.logR, ps.Ns);
+    return n;
+}
+
+template <int LOGR>
+static void init_pass_tw(const fc2_plan_s* p, cpx<double>* tab, int logD, cudaStream_t s) {
+    constexpr int LOGJ = FftCfg<double>::LOGE - LOGR, Q = 1 << stage_bits(LOGR, 0);
+    const int64_t nb = (pass_tw_tiles(logD, LOGJ) << FftCfg<double>::LOGE) / Q;
+    k_init_pass_tw<LOGR, LOGJ><<<(unsigned)((nb + 255) / 256), 256, 0, s>>>(
+        tab, p->logM, logD, (const cpx<double>*)p->d_twlo, (const cpx<double>*)p->d_twhi, p->tw_shift);
+}
+
 cudaError_t init_twiddles(fc2_plan_s* p, cudaStream_t s) {
     int sh;
     int64_t nlo, nhi;
@@ -1931,6 +2021,26 @@ cudaError_t init_twiddles(fc2_plan_s* p, cudaStream_t s) {
     else
         k_init_tw<float><<<blocks, 256, 0, s>>>((cpx<float>*)p->d_twlo, nlo,
                                                 (cpx<float>*)p->d_twhi, nhi, p->logM, sh);
+    if (p->d_twpass) {
+        cpx<double>* tab = (cpx<double>*)p->d_twpass;
+        for (const auto& ps : p->passes) {
+            const int64_t n = pass_tw_entries(p->logM, ps.logR, ps.Ns);
+            if (n == 0) continue;
+            int logD = 0;
+            while ((1ll << logD) < ps.Ns) ++logD;
+            switch (ps.logR) {
+                case 5: init_pass_tw<5>(p, tab, logD, s); break;
+                case 6: init_pass_tw<6>(p, tab, logD, s); break;
+                case 7: init_pass_tw<7>(p, tab, logD, s); break;
+                case 8: init_pass_tw<8>(p, tab, logD, s); break;
+                case 9: init_pass_tw<9>(p, tab, logD, s); break;
+                case 10: init_pass_tw<10>(p, tab, logD, s); break;
+                case 11: init_pass_tw<11>(p, tab, logD, s); break;
+                default: return cudaErrorInvalidValue;
+            }
+            tab += n;
+        }
+    }
     return cudaGetLastError();
 }
 
@@ -2250,17 +2360,23 @@ static cudaError_t run_pass(fc2_plan_s* p, const void* in, void* out, const Pass
     return cudaGetLastError();
 }
 
-template <int LOGR>
+template <int LOGR, bool FUSED>
 static cudaError_t run_pass_d(fc2_plan_s* p, const void* in, void* out, const PassArgs& a,
                               cudaStream_t s) {
     constexpr int LOGJ = FftCfg<double>::LOGE - LOGR, NT = FftCfg<double>::NT;
     constexpr size_t smem = (size_t)(phys((1 << FftCfg<double>::LOGE) - 1) + 1) * sizeof(cpx<double>);
-    auto kern = k_fft_pass_d<LOGR, LOGJ, NT>;
+    auto kern = k_fft_pass_d<LOGR, LOGJ, NT, FUSED>;
     const cudaError_t e = raise_smem_limit((const void*)kern, smem);
     if (e != cudaSuccess) return e;
     dim3 grid((unsigned)((p->M >> LOGR) >> LOGJ), (unsigned)a.ng);
-    kern<<<grid, NT, smem, s>>>((const cpx<double>*)in, (cpx<double>*)out, a, p->d_L,
-                                (const cpx<double>*)p->d_twlo);
+    const cpx<double>* tw = (const cpx<double>*)(FUSED ? p->d_twlo : p->d_twpass);
+    if (!FUSED)
+        for (const auto& ps : p->passes) {  // the tables of the passes before this one
+            if (ps.Ns == (1ll << a.logNs)) break;
+            tw += pass_tw_entries(p->logM, ps.logR, ps.Ns);
+        }
+    kern<<<grid, NT, smem, s>>>((const cpx<double>*)in, (cpx<double>*)out, a, p->d_L, tw,
+                                (const cpx<double>*)p->d_twst + p->twst_off[LOGR]);
     return cudaGetLastError();
 }
 
@@ -2374,12 +2490,12 @@ static cudaError_t run_radix(fc2_plan_s* p, const void* in, void* out, const Pas
     // Batches return float, where the fused kernel's other rounding is far below
     // an ulp; a plan returns double Delta chi^2, and its bins of coefficient norm
     // up to 1e7 would carry a change of rounding to 3e-7 of the rms, so plans keep
-    // the operation order of k_fft_pass (the fused kernel would take a
-    // 2^20-bin plan of four harmonics from 6.5 to 5.2 ms).
+    // the operation order (the fused kernel would take a 2^20-bin plan of four
+    // harmonics from 6.5 to 5.2 ms).
     if constexpr (sizeof(T) == 8 && LOGJ >= 0) {
-        if (p->fused_fft) return run_pass_d<LOGR>(p, in, out, a, s);
-    }
-    if constexpr (LOGJ >= 0) return run_pass<T, LOGR, LOGJ, FftCfg<T>::NT>(p, in, out, a, s);
+        return p->fused_fft ? run_pass_d<LOGR, true>(p, in, out, a, s)
+                            : run_pass_d<LOGR, false>(p, in, out, a, s);
+    } else if constexpr (LOGJ >= 0) return run_pass<T, LOGR, LOGJ, FftCfg<T>::NT>(p, in, out, a, s);
     return cudaErrorInvalidValue;
 }
 

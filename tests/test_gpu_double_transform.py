@@ -32,3 +32,21 @@ def test_fp64_batch_matches_oracle(oracle_mod, N, fill):
         _, _, chi0, _ = oracle_mod.moments(cur.x, cur.sigma)
         ok = piv >= 1e-6  # sums good to 1e-12 against pivots above 1e-6
         assert np.max(np.abs(blk[:, bins].T - ref)[ok], initial=0.0) <= 1e-5 * chi0
+
+
+@pytest.mark.parametrize("N,fill", [(2048, 0.3), (6001, 0.02), (16384, 0.4), (30011, 0.1), (65536, 0.05),
+                                    (131072, 0.2), (262144, 0.45), (524288, 0.03), (1048576, 0.1),
+                                    (2000001, 0.3), (8388608, 0.02)])
+def test_fp64_plan_matches_oracle(oracle_mod, N, fill):
+    """Plans keep the passes' operation order, with tabled inter-pass twiddles
+    and skipped zeros (2^12 .. 2^24 points, two and three passes)."""
+    from paper_0901_1913_gb300 import _fc2
+    c = synth.short_curve(seed=N % 89, n=80)
+    H, df = 2, fill / 100.0
+    f_min = 0.31 * df + 0.03
+    d, _, _, chi0 = _fc2.periodogram(c.t, c.x, c.sigma, H, f_min, df, N, 2, "fp64")
+    bins = np.unique(np.concatenate([np.random.default_rng(N).integers(0, N, 150),
+                                     [0, 1, N // 2 - 1, N // 2, N - 2, N - 1]]))
+    ref, piv = oracle_mod.dchi2_bins(c.t, c.x, c.sigma, H, f_min, df, bins, with_pivots=True)
+    ok = piv >= 1e-4  # sums good to 1e-11 of W (phases up to 1e5 turns) against such pivots
+    assert np.max(np.abs(d[:, bins].T - ref)[ok], initial=0.0) <= 1e-6 * chi0
