@@ -658,6 +658,42 @@ __global__ void __launch_bounds__(PK_NT) k_peaks1(const double* __restrict__ d, 
     }
 }
 
+// The same with one CTA per block and task (rows 0..H-1, then the local maxima):
+// a short trial grid's few blocks waited on their loads row after row.
+// N = 2^20, H = 6 (256 blocks): 52 -> 23 us; N = 16384, H = 3: 18 -> 9 us; equal at
+// 1024 blocks; slower for long grids (8192 blocks, H = 8: 638 against 560 us),
+// which k_peaks1 keeps: PK_SPLIT blocks x tasks at most.
+constexpr int64_t PK_SPLIT = 32 * 152;
+__global__ void __launch_bounds__(PK_NT) k_peaks1_split(const double* __restrict__ d, int64_t N, int H,
+                                                        Cand* __restrict__ amax,
+                                                        Cand* __restrict__ bmax, int nblk) {
+    __shared__ Cand wres[PK_NW];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int64_t base = (int64_t)blockIdx.x * PK_B;
+    const bool maxima = (int)blockIdx.y == H;
+    const double* row = d + (int64_t)(maxima ? H - 1 : blockIdx.y) * N;
+    int64_t v = KEY_NONE, j = INT64_MAX;
+#pragma unroll
+    for (int q = 0; q < PK_PER; ++q) {
+        const int64_t jj = base + threadIdx.x + (int64_t)q * PK_NT;
+        if (jj < N) {
+            const int64_t x = okey(row[jj]);
+            const bool ok = !maxima || ((jj == 0 || x > okey(row[jj - 1])) &&
+                                        (jj == N - 1 || x >= okey(row[jj + 1])));
+            if (ok && better(x, jj, v, j)) { v = x; j = jj; }
+        }
+    }
+    warp_best(v, j);
+    if (lane == 0) wres[w] = Cand{v, j};
+    __syncthreads();
+    if (w == 0) {
+        v = lane < PK_NW ? wres[lane].k : KEY_NONE;
+        j = lane < PK_NW ? wres[lane].j : INT64_MAX;
+        warp_best(v, j);
+        if (lane == 0) (maxima ? bmax : amax + (int64_t)blockIdx.y * nblk)[blockIdx.x] = Cand{v, j};
+    }
+}
+
 // Block-wide best of (v, j) over the CTA (blockDim.x <= 1024); every thread
 // gets the winner.
 FC2_D Cand block_best(int64_t v, int64_t j, Cand* ws) {
@@ -972,7 +1008,11 @@ cudaError_t launch_peaks(fc2_plan_s* p, cudaStream_t s) {
     int32_t* ncand = (int32_t*)(theta + 1);
     Cand* cand = theta + 2;
     int64_t* rec_j = (int64_t*)(cand + cap);
-    k_peaks1<<<(unsigned)nblk, PK_NT, 0, s>>>(p->d_dchi2, p->N, H, amax, bmax, (int)nblk);
+    if (nblk * (H + 1) <= PK_SPLIT)
+        k_peaks1_split<<<dim3((unsigned)nblk, (unsigned)(H + 1)), PK_NT, 0, s>>>(
+            p->d_dchi2, p->N, H, amax, bmax, (int)nblk);
+    else
+        k_peaks1<<<(unsigned)nblk, PK_NT, 0, s>>>(p->d_dchi2, p->N, H, amax, bmax, (int)nblk);
     k_peaks2<<<1, 1024, 0, s>>>(amax, bmax, (int)nblk, H, K, rec_j, theta, ncand);
     k_peaks3<<<(unsigned)nblk, PK_NT, 0, s>>>(p->d_dchi2, p->N, H, bmax, theta, cand, ncand, cap);
     k_peaks4<<<1, 1024, 0, s>>>(cand, ncand, cap, K, rec_j + H);
