@@ -450,6 +450,7 @@ fc2_status fc2_plan_create(const double* t, const double* x, const double* sigma
             const double c = (double)gg.k * df;
             const double pmax = c * p->scal[SC_TAUMAX];
             const double cells = pmax * (double)M;
+            gg.turns = pmax;
             if (!(pmax < 1.0) || cells + wg + 2.0 >= (double)M) {
                 gg.wraps = (pmax >= 1.0) ? 1 : 0;
                 gg.L = M;
@@ -524,9 +525,12 @@ static int64_t launches_front(const fc2_plan_s* p) {
     int64_t n = 1 + 1 + (int64_t)p->passes.size() + 1 + (p->fp64 ? 0 : 1);  // phase, spread, fft, assemble(+resolve)
     int bits = 0;
     while ((1ll << bits) < p->M + 2 * std::max(p->w, p->w_p) + 2) ++bits;
-    int64_t wraps = 0;
-    for (auto& g : p->geom) wraps += g.wraps ? 1 : 0;
-    if (wraps > 0) n += p->n <= RUN_CAP ? 1 : wraps * (2 + 3 * ((bits + 7) / 8));
+    bool runs = false;
+    for (auto& g : p->geom) {
+        if (g.by_runs(p->n)) runs = true;
+        else if (g.wraps) n += 2 + 3 * ((bits + 7) / 8);
+    }
+    if (runs) ++n;
     return n;
 }
 

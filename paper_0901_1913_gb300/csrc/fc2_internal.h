@@ -64,14 +64,25 @@ inline int fft_family_of(int fft_kernel) {
 }
 
 // Longest sample set whose wrapping keys are ordered by its runs in one launch
-// (k_sort_runs); longer ones take the radix sort.
+// (k_sort_runs), and the most samples x runs, since every sample is placed against
+// every run (at most one run per sample).  Other sets take the radix sort: some
+// 90 us a set, which the line keeps one set's run ordering below.  One-shot calls
+// of three wrapping sets by radix and by runs, 7168 samples: 895 and 628 us at 1.6
+// turns, 793 at 32, 1177 at 128, 4061 at 2048; 2000 samples: 785 and 504, 539, 618,
+// 844; 500 samples: 725 and 452 to 488 at any number of turns.
 constexpr int RUN_CAP = 7168;
+constexpr double RUN_WORK = 262144.0;
 
 struct GridGeom {
     int k;            // harmonic multiple of this transform
     int kind;         // 0 = Q (weights), 1 = P (weighted data)
     int64_t L;        // occupied extent in cells (rows beyond are zero)
     int wraps;        // samples wrap the fold period -> keys need sorting
+    double turns;     // of the fold over the samples
+    // keys ordered by k_sort_runs (n samples)
+    bool by_runs(int64_t n) const {
+        return wraps && n <= RUN_CAP && n * (turns < n ? turns : (double)n) <= RUN_WORK;
+    }
 };
 
 struct FftPass {

@@ -2014,6 +2014,7 @@ fc2_status batched_execute(int64_t C, const int64_t* offsets, const double* t, c
                 const double cells = pmax * (double)M;
                 GridGeom& gg = p.geom[gi];
                 gg.k = k; gg.kind = kind;
+                gg.turns = pmax;
                 if (!(pmax < 1.0) || cells + p.w + 2.0 >= (double)M) {
                     gg.wraps = (pmax >= 1.0) ? 1 : 0;
                     cellsv.push_back(-1.0);

@@ -705,8 +705,9 @@ static cudaError_t sort_keys_of(fc2_plan_s* p, int g, cudaStream_t s) {
 // The radix sort takes five to eleven launches and three copies a set, each
 // shorter than its launch: 16 wrapping sets of some 500 samples spent 430 us in
 // it, 5 us here (the batched call of their 12 curves 1.89 -> 1.00 ms, a short
-// double session with five such sets 1.27 -> 1.00 ms).  Longer sets (more steps
-// of one CTA than launches saved) stay with the radix sort.
+// double session with five such sets 1.27 -> 1.00 ms).  Longer sets and those of
+// many turns (more steps of one CTA than launches saved: GridGeom::by_runs) stay
+// with the radix sort; here they are in order already, one run.
 constexpr int RUN_NT = 1024;
 template <typename T>
 __global__ void __launch_bounds__(RUN_NT) k_sort_runs(int32_t* key, T* dlt, cpx<T>* cs, int64_t n_all,
@@ -780,14 +781,14 @@ static cudaError_t sort_wrapping_impl(fc2_plan_s* p, cudaStream_t s) {
     for (int g = 0; g < nset; ++g) {
         const int64_t n = per_slot ? p->h_slot_n[g] : p->n;
         total = std::max(total, (per_slot ? p->h_slot_soff[g] : (int64_t)g * p->n) + n);
-        small = small || (p->geom[g].wraps && n <= RUN_CAP);
+        small = small || p->geom[g].by_runs(n);
     }
     // the sorted copies go to the second grid buffer, free until the spread
     const size_t need = (size_t)total * (4 + 3 * sizeof(T)) + 512;
     const bool runs = small && need <= (size_t)p->G * (size_t)p->M * sizeof(cpx<T>);
     for (int g = 0; g < nset; ++g) {
         const int64_t n = per_slot ? p->h_slot_n[g] : p->n;
-        if (p->geom[g].wraps && !(runs && n <= RUN_CAP)) {
+        if (p->geom[g].wraps && !(runs && p->geom[g].by_runs(n))) {
             const cudaError_t e = sort_keys_of<T>(p, g, s);
             if (e != cudaSuccess) return e;
         }

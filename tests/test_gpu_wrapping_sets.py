@@ -1,5 +1,5 @@
 """Sample sets whose fold wraps, at lengths around the run ordering's block and
-its cap (longer sets take the radix sort), over one to many turns, in both
+its cap (longer sets, and those of many turns, take the radix sort), in both
 precisions and in a batch of mixed lengths, against the oracle."""
 import numpy as np
 import pytest
@@ -20,7 +20,8 @@ def check(oracle_mod, c, H, N, f_min, df, d):
 
 @pytest.mark.parametrize("prec", ["mixed", "fp64"])
 @pytest.mark.parametrize("n,turns", [(40, 40.0), (1023, 0.7), (1024, 1.6), (1025, 3.3), (2048, 9.2),
-                                     (7167, 1.1), (7168, 2.4), (7169, 2.4)])
+                                     (7167, 1.1), (7168, 2.4), (7169, 2.4),
+                                     (700, 93.0), (3000, 400.0)])
 def test_plan_matches_oracle(oracle_mod, prec, n, turns):
     from paper_0901_1913_gb300 import _fc2
     c = synth.short_curve(seed=n, n=n)
