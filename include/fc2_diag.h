@@ -78,6 +78,13 @@ void fc2_debug_fail_alloc(int64_t k);
  * process (including those fc2_debug_fail_alloc made fail). */
 int64_t fc2_debug_alloc_count(void);
 
+/* The free device memory (bytes) assumed when a double-precision call decides
+ * whether the twiddle tables of its transform passes fit (they are allocated
+ * where they take at most an eighth of what the call leaves over; without
+ * them the passes form the twiddles).  0 asks the device again.  Process-wide;
+ * for tests. */
+void fc2_debug_table_memory(int64_t bytes);
+
 /* Bytes of the library's device pool on `device` in use by live allocations,
  * after waiting for all work on the device (0 if the library never allocated
  * there, -1 on a CUDA error). */

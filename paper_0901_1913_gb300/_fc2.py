@@ -164,6 +164,8 @@ def load():
         lib.fc2_debug_last_tier.restype = None
         lib.fc2_debug_fail_alloc.argtypes = [i64]
         lib.fc2_debug_fail_alloc.restype = None
+        lib.fc2_debug_table_memory.argtypes = [i64]
+        lib.fc2_debug_table_memory.restype = None
         lib.fc2_debug_alloc_count.argtypes = []
         lib.fc2_debug_alloc_count.restype = i64
         lib.fc2_debug_pool_used.argtypes = [i32]
@@ -428,6 +430,12 @@ def spread_force_general(on=True):
     default, where tiles of one sample set that fit one staging batch go to
     the single-batch kernel (False)."""
     load().fc2_debug_spread_force_general(int(bool(on)))
+
+
+def table_memory(nbytes=0):
+    """Free device memory assumed when a double-precision call decides whether
+    its transform's twiddle tables fit (0: ask the device)."""
+    load().fc2_debug_table_memory(int(nbytes))
 
 
 def trim_device_memory(device=0):

@@ -80,6 +80,30 @@ static cudaMemPool_t existing_pool(int dev) {
     auto it = g_pools.find(dev);
     return it == g_pools.end() ? nullptr : it->second;
 }
+
+// Tables that only save time are allocated where they take at most an eighth of
+// the memory a call leaves over: near the device's limit a call that fits
+// without them still fits.  `need`: the call's own estimate; memory the pool
+// holds unused counts as free.
+static std::atomic<int64_t> g_table_memory{0};  // fc2_debug_table_memory
+bool table_room(size_t bytes, size_t need) {
+    size_t avail = 0, total = 0;
+    const int64_t forced = g_table_memory.load();
+    int dev = 0;
+    if (forced > 0) {
+        avail = (size_t)forced;
+    } else if (cudaGetDevice(&dev) != cudaSuccess || cudaMemGetInfo(&avail, &total) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    } else if (cudaMemPool_t pool = existing_pool(dev)) {
+        uint64_t held = 0, used = 0;
+        if (cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, &held) == cudaSuccess &&
+            cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemCurrent, &used) == cudaSuccess)
+            avail += held - std::min(held, used);
+        cudaGetLastError();
+    }
+    return avail > need && bytes <= (avail - need) / 8;
+}
 }  // namespace fc2
 
 namespace {
@@ -245,12 +269,8 @@ fc2_status fc2_plan_create(const double* t, const double* x, const double* sigma
     const int NSRC = p->nsrc ? p->nsrc : G;  // sample sets
     const size_t spec_rows = p->packed ? (size_t)2 * G : (size_t)G;
     const size_t spec_bytes = p->paper ? (size_t)M * csz : spec_rows * N * csz;
-    // with the autotuner the passes may change: room for any plan's tables (each
-    // pass after the first needs at most the grid length, or one tile)
-    const int64_t tw_pass = !p->fp64 ? 0 : (opt.autotune > 0 ? 4 * std::max<int64_t>(M, 4096)
-                                                             : plan_pass_tw_entries(p));
     // memory estimate
-    size_t need = (size_t)tw_pass * csz;
+    size_t need = 0;
     need += (size_t)n * 8 * 6 + (size_t)n * 4;
     need += (size_t)NSRC * n * (4 + tsz + csz);
     need += 2 * (size_t)G * M * csz;
@@ -261,6 +281,10 @@ fc2_status fc2_plan_create(const double* t, const double* x, const double* sigma
         delete p;
         return FC2_ERR_OOM;
     }
+    // inter-pass twiddle tables of double plans (with the autotuner the passes may
+    // change: the most any candidate needs), where there is room for them
+    int64_t tw_pass = plan_pass_tw_entries(p, opt.autotune > 0);
+    if (tw_pass > 0 && !table_room((size_t)tw_pass * csz, need)) tw_pass = 0;
 
     Guard g;
     if (opt.inputs_on_device) {
@@ -787,6 +811,8 @@ fc2_status fc2_debug_spectra(fc2_plan p, double* re, double* im) {
 double fc2_debug_t0(fc2_plan p) { return p ? p->scal[SC_T0] : 0.0; }
 
 void fc2_debug_last_tier(int tier) { set_last_fixup_tier(tier); }
+
+void fc2_debug_table_memory(int64_t bytes) { g_table_memory.store(bytes > 0 ? bytes : 0); }
 
 void fc2_debug_fail_alloc(int64_t k) { g_fail_alloc_in.store(k > 0 ? k : 0); }
 

@@ -157,11 +157,11 @@ struct fc2_plan_s {
     void* d_twhi = nullptr;
     int tw_shift = 0;
     void* d_twst = nullptr;    // cpx<T> in-CTA stage twiddles per radix
-    void* d_twpass = nullptr;  // double plans: inter-pass twiddles in tile order
+    void* d_twpass = nullptr;  // double plans: inter-pass twiddles in tile order (null: formed)
     int64_t twst_off[16] = {0};
     int64_t tw64_off[16] = {0};
     int fft_family = fc2::FFT_R64;  // kernel family of the float passes (fc2::FftFamily)
-    bool fused_fft = false;    // double passes by k_fft_pass_d (batches, whose results are float)
+    bool fused_fft = false;    // double passes in k_fft_pass_d's fused form (batches, whose results are float)
     int fft_group = 0;         // grids taken through all passes together (0 = all)
     int spread_tile = 0;       // cells per spreading tile (0 = default for M)
     double* d_dchi2 = nullptr; // [H][N]
@@ -254,7 +254,7 @@ cudaError_t launch_detrend(const double* t, const double* x, const double* sigma
 
 // k_fft.cu
 void twiddle_split(int logM, bool fused, int* sh, int64_t* nlo, int64_t* nhi);  // d_twlo, d_twhi entries
-int64_t plan_pass_tw_entries(const fc2_plan_s* p);  // d_twpass entries (0: none)
+int64_t plan_pass_tw_entries(const fc2_plan_s* p, bool tuned);  // d_twpass entries (0: none)
 cudaError_t init_twiddles(fc2_plan_s* p, cudaStream_t s);
 cudaError_t init_deconv(fc2_plan_s* p, cudaStream_t s);
 void plan_fft_passes(fc2_plan_s* p);
@@ -271,6 +271,7 @@ void forget_batch_tuning();
 void force_batch_config(int spread_tile, int asm_nt, int bx_ch, int fft_group);
 void force_batch_plan(const int* rs, int n, int family);
 cudaError_t pool_alloc(void** ptr, size_t bytes, cudaStream_t s);  // library device pool
+bool table_room(size_t bytes, size_t need);  // whether optional tables are allocated
 void drop_deconv_cache(int dev);  // k_fft.cu: cached deconvolution tables of a device
 cudaError_t launch_fft(fc2_plan_s* p, cudaStream_t s);
 

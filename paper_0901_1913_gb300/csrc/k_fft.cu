@@ -1964,12 +1964,6 @@ static int64_t pass_tw_entries(int logM, int logR, int64_t Ns) {
     while ((1ll << logD) < Ns) ++logD;
     return pass_tw_tiles(logD, FftCfg<double>::LOGE - logR) << FftCfg<double>::LOGE;
 }
-int64_t plan_pass_tw_entries(const fc2_plan_s* p) {
-    int64_t n = 0;
-    if (p->fp64 && !p->fused_fft)
-        for (const auto& ps : p->passes) n += pass_tw_entries(p->logM, ps.logR, ps.Ns);
-    return n;
-}
 
 template <int LOGR>
 static void init_pass_tw(const fc2_plan_s* p, cpx<double>* tab, int logD, cudaStream_t s) {
@@ -2162,6 +2156,26 @@ static std::vector<std::vector<int>> fft_candidates(int logM, int maxr) {
     const std::vector<int> more = balanced_split(logM, P + 1);
     if (more.back() >= 8) out.push_back(more);
     return out;
+}
+
+// Entries of a double plan's inter-pass twiddle tables: those of its own passes,
+// or with the autotuner of whichever candidate needs most.
+int64_t plan_pass_tw_entries(const fc2_plan_s* p, bool tuned) {
+    if (!p->fp64 || p->fused_fft) return 0;
+    auto entries = [&](const std::vector<int>& rs) {
+        int64_t n = 0, Ns = 1;
+        for (int r : rs) {
+            n += pass_tw_entries(p->logM, r, Ns);
+            Ns <<= r;
+        }
+        return n;
+    };
+    std::vector<int> own;
+    for (const auto& ps : p->passes) own.push_back(ps.logR);
+    int64_t n = entries(own);
+    if (tuned)
+        for (const auto& rs : fft_candidates(p->logM, FftCfg<double>::MAXR)) n = std::max(n, entries(rs));
+    return n;
 }
 
 struct TuneKey {
@@ -2492,10 +2506,13 @@ static cudaError_t run_radix(fc2_plan_s* p, const void* in, void* out, const Pas
     // up to 1e7 would carry a change of rounding to 3e-7 of the rms, so plans keep
     // the operation order (the fused kernel would take a 2^20-bin plan of four
     // harmonics from 6.5 to 5.2 ms).
+    // A double call whose tables did not fit (table_room) runs k_fft_pass, which
+    // forms the twiddles.
     if constexpr (sizeof(T) == 8 && LOGJ >= 0) {
-        return p->fused_fft ? run_pass_d<LOGR, true>(p, in, out, a, s)
-                            : run_pass_d<LOGR, false>(p, in, out, a, s);
-    } else if constexpr (LOGJ >= 0) return run_pass<T, LOGR, LOGJ, FftCfg<T>::NT>(p, in, out, a, s);
+        if (p->fused_fft) return run_pass_d<LOGR, true>(p, in, out, a, s);
+        if (a.first || p->d_twpass) return run_pass_d<LOGR, false>(p, in, out, a, s);
+    }
+    if constexpr (LOGJ >= 0) return run_pass<T, LOGR, LOGJ, FftCfg<T>::NT>(p, in, out, a, s);
     return cudaErrorInvalidValue;
 }
 
