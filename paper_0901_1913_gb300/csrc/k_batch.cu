@@ -1715,7 +1715,8 @@ fc2_status batched_execute(int64_t C, const int64_t* offsets, const double* t, c
             const size_t bytes = (size_t)(ch.S + sl) * (size_t)ch.M * csz * 2 +
                                  (size_t)(ch.S + sl) * ch.N * csz +
                                  (size_t)(ch.slot_samples + sl * n) * (4 + tsz + csz) +
-                                 (size_t)(ch.ntot + n) * 80;
+                                 (size_t)(ch.ntot + n) * 80 +
+                                 (fp64 ? (size_t)(ch.M / 2) * csz : 0);  // fused twiddles
             if (ch.c1 > a && bytes > budget) break;
             ch.S += sl;
             ch.ntot += n;
@@ -1867,7 +1868,13 @@ fc2_status batched_execute(int64_t C, const int64_t* offsets, const double* t, c
             release(p.d_twlo, s); release(p.d_twhi, s); release(p.d_twst, s); release(p.d_dec, s);
             int sh;
             int64_t nlo, nhi;
-            p.fused_fft = fp64;
+            // the fused double passes keep M / 2 twiddles; near the memory's limit the
+            // general pass forms them instead (the first chunk's buffers are still
+            // to be allocated, at the largest size any chunk needs)
+            p.fused_fft = fp64 && table_room((size_t)(M / 2) * csz,
+                                             b.grid0 ? 0 : 2 * mx_grid + mx_spec +
+                                                           (size_t)mx.slot_samples * (4 + tsz + csz) +
+                                                           (size_t)mx.ntot * 80);
             twiddle_split(p.logM, p.fused_fft, &sh, &nlo, &nhi);
             cudaError_t ea = pool_alloc((void**)&p.d_twlo, (size_t)nlo * csz, s);
             if (ea == cudaSuccess) ea = pool_alloc((void**)&p.d_twhi, (size_t)nhi * csz, s);

@@ -57,3 +57,29 @@ def test_plan_without_tables_gives_the_same_values(N):
             _fc2.table_memory(0)
     np.testing.assert_array_equal(S[0][0], S[1][0])
     np.testing.assert_array_equal(S[0][1], S[1][1])
+
+
+@pytest.mark.parametrize("N", [2048, 6001, 1 << 15, 1 << 18])
+def test_batch_without_tables_matches_oracle(oracle_mod, N):
+    from paper_0901_1913_gb300 import _fc2
+    b = synth.survey_batch(seed=N % 97, C=3, N=N, T=50.0, f_max=1.0, n_median=60.0, n_hi=120)
+    Hs = np.array([1, 2, 3], dtype=np.int32)
+    df, f_min = 0.0013, 0.0604
+    _fc2.table_memory(1)
+    try:
+        d, _, _ = _fc2.execute_batched(b.offsets, b.t, b.x, b.sigma, Hs, f_min, df, N, 2, "fp64",
+                                       autotune="fixed")
+    finally:
+        _fc2.table_memory(0)
+    bins = np.unique(np.concatenate([np.random.default_rng(N).integers(0, N, 120), [0, N - 1]]))
+    at = 0
+    for c in range(3):
+        cur, H = b.curve(c), int(Hs[c])
+        blk = d[at:at + H * N].reshape(H, N)
+        at += H * N
+        ref, piv = oracle_mod.dchi2_bins(cur.t, cur.x, cur.sigma, H, f_min, df, bins, with_pivots=True)
+        _, _, chi0, _ = oracle_mod.moments(cur.x, cur.sigma)
+        ok = piv >= 1e-4
+        assert ok.sum() > 30
+        # sums good to 1e-12 of W against such pivots, then a float result
+        assert np.max(np.abs(blk[:, bins].T - ref)[ok]) <= 1e-6 * chi0
