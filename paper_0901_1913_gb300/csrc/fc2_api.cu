@@ -83,26 +83,25 @@ static cudaMemPool_t existing_pool(int dev) {
 
 // Tables that only save time are allocated where they take at most an eighth of
 // the memory a call leaves over: near the device's limit a call that fits
-// without them still fits.  `need`: the call's own estimate; memory the pool
-// holds unused counts as free.
+// without them still fits.  `need`: the call's own estimate; `freeb`: the
+// device's free memory (the caller has asked for it), to which the memory the
+// pool holds unused is added.
 static std::atomic<int64_t> g_table_memory{0};  // fc2_debug_table_memory
-bool table_room(size_t bytes, size_t need) {
-    size_t avail = 0, total = 0;
+bool table_room(size_t bytes, size_t need, size_t freeb) {
     const int64_t forced = g_table_memory.load();
     int dev = 0;
     if (forced > 0) {
-        avail = (size_t)forced;
-    } else if (cudaGetDevice(&dev) != cudaSuccess || cudaMemGetInfo(&avail, &total) != cudaSuccess) {
-        cudaGetLastError();
-        return false;
-    } else if (cudaMemPool_t pool = existing_pool(dev)) {
-        uint64_t held = 0, used = 0;
-        if (cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, &held) == cudaSuccess &&
-            cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemCurrent, &used) == cudaSuccess)
-            avail += held - std::min(held, used);
+        freeb = (size_t)forced;
+    } else if (cudaGetDevice(&dev) == cudaSuccess) {
+        if (cudaMemPool_t pool = existing_pool(dev)) {
+            uint64_t held = 0, used = 0;
+            if (cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, &held) == cudaSuccess &&
+                cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemCurrent, &used) == cudaSuccess)
+                freeb += held - std::min(held, used);
+        }
         cudaGetLastError();
     }
-    return avail > need && bytes <= (avail - need) / 8;
+    return freeb > need && bytes <= (freeb - need) / 8;
 }
 }  // namespace fc2
 
@@ -284,7 +283,7 @@ fc2_status fc2_plan_create(const double* t, const double* x, const double* sigma
     // inter-pass twiddle tables of double plans (with the autotuner the passes may
     // change: the most any candidate needs), where there is room for them
     int64_t tw_pass = plan_pass_tw_entries(p, opt.autotune > 0);
-    if (tw_pass > 0 && !table_room((size_t)tw_pass * csz, need)) tw_pass = 0;
+    if (tw_pass > 0 && !table_room((size_t)tw_pass * csz, need, freeb)) tw_pass = 0;
 
     Guard g;
     if (opt.inputs_on_device) {

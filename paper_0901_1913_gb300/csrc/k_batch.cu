@@ -1869,12 +1869,12 @@ fc2_status batched_execute(int64_t C, const int64_t* offsets, const double* t, c
             int sh;
             int64_t nlo, nhi;
             // the fused double passes keep M / 2 twiddles; near the memory's limit the
-            // general pass forms them instead (the first chunk's buffers are still
-            // to be allocated, at the largest size any chunk needs)
+            // general pass forms them instead
             p.fused_fft = fp64 && table_room((size_t)(M / 2) * csz,
-                                             b.grid0 ? 0 : 2 * mx_grid + mx_spec +
-                                                           (size_t)mx.slot_samples * (4 + tsz + csz) +
-                                                           (size_t)mx.ntot * 80);
+                                             2 * mx_grid + mx_spec +
+                                                 (size_t)mx.slot_samples * (4 + tsz + csz) +
+                                                 (size_t)mx.ntot * 80,
+                                             freeb);
             twiddle_split(p.logM, p.fused_fft, &sh, &nlo, &nhi);
             cudaError_t ea = pool_alloc((void**)&p.d_twlo, (size_t)nlo * csz, s);
             if (ea == cudaSuccess) ea = pool_alloc((void**)&p.d_twhi, (size_t)nhi * csz, s);
