@@ -122,15 +122,27 @@ fc2_status fc2_debug_exact_bins(fc2_plan p, const int64_t* bins, int64_t nb, int
  * the grid, and each next pass's tile width is at most the current radix);
  * otherwise (or with validate = 0) the host replay of the kernels' index
  * arithmetic for that plan -- the global loads of each pass's input, the
- * stores toward the next pass on each kernel's store path, the shared tile
- * slots those stores read, the inter-pass twiddle exponents -- over the
- * first, last and spread tiles of every pass: 0 when all are in range, else
- * 100 * (pass + 1) + the failing check, with info4 (may be NULL) = pass,
- * check, tile, index.  -1 on bad arguments. */
+ * stores toward the next pass on the route its kernel takes, the shared tile
+ * slots those stores read, the inter-pass twiddle exponents and table
+ * entries -- over the first, last and spread tiles of every pass: 0 when all
+ * are in range and every store goes where the next pass reads that output,
+ * else 100 * (pass + 1) + the failing check, with info4 (may be NULL) = pass,
+ * check, tile, index.  -1 on bad arguments.
+ *
+ * fc2_debug_fft_pass: what launches pass `pass` (and what the replay follows):
+ * out4 = kernel (0 whole transform, 1 radix-16 stages, 2 register stages of
+ * radix 64, 3 bulk copies, 4 register stages of radix 32, 5 bulk copies by two
+ * groups, 6 the 2^10 first pass by three groups, 7 double), log2 of a tile's
+ * columns, threads that store a tile, route of its stores (0 modes of a last
+ * pass, 1 rows of a two-pass plan, 2 one stride per thread, 3 element by
+ * element, 4 straight from registers).  1 for a plan the kernels refuse, -1 on
+ * bad arguments. */
 int fc2_debug_fft_plan(int logM, int fp64, int* radices, int max_passes);
 int fc2_debug_fft_candidates(int logM, int fp64, int* radices, int max_entries);
 int fc2_debug_fft_plan_check(int logM, int fp64, int fft_kernel, const int* radices, int P,
                              int validate, int64_t* info4);
+int fc2_debug_fft_pass(int logM, int fp64, int fft_kernel, const int* radices, int P, int pass,
+                       int* out4);
 
 /* Kernels launched by the last fc2_execute_batched call of this process. */
 int64_t fc2_debug_batch_launches(void);

@@ -35,9 +35,10 @@ constexpr size_t DFTAB_BYTES = (size_t)(DFTAB_T16 + 65536) * 16;
 // Float transform kernel families (double passes always use FFT_R16).
 enum FftFamily {
     FFT_R16 = 0,   // radix-16 stages in shared memory (k_fft_pass)
-    FFT_R64 = 1,   // two register stages of radix R/64 and 64 (k_fft_pass64) for radix
-                   // 2^10..2^12, FFT_BULK's kernel for 2^8 and 2^9
-    FFT_BULK = 2,  // radix-16 stages fed by bulk asynchronous copies (k_fft_pass_tma), 2^8..2^12
+    FFT_R64 = 1,   // two register stages of radix R/64 and 64 for radix 2^10..2^12
+                   // (k_fft_pass64; a first 2^10 pass k_fft_first10), FFT_BULK's for 2^8 and 2^9
+    FFT_BULK = 2,  // stages fed by bulk asynchronous copies (k_fft_pass_duo for 2^8 and 2^9,
+                   // k_fft_pass_tma for 2^10..2^12)
     FFT_R32 = 3,   // two register stages of radix 32 and 32 (k_fft_pass32, 512 threads) for
                    // radix 2^10; FFT_BULK's kernel for 2^8, 2^9, 2^11 and 2^12
     FFT_R32X = 4   // k_fft_pass32 for radix 2^9 (16 x 32) and 2^10; FFT_BULK's kernel for

@@ -447,6 +447,22 @@ struct PassArgs {
     int g0, ng;        // this launch covers grids g0 .. g0 + ng - 1
 };
 
+// Which way a pass stores towards the next one; the kernels and the host replay
+// ask the same predicates.
+// A two-pass plan: output k of column j is row j, column k of the last pass.
+FC2_HD bool two_pass(const PassArgs& a, int LOGR) { return a.logNs == 0 && a.logM - a.logRn == LOGR; }
+// store_tile_blocked's one-stride form.
+FC2_HD bool one_stride(const PassArgs& a, int LOGR, int LOGJ, int NT) {
+    return a.logNs == 0 && LOGR <= a.logM - a.logRn && a.logJn <= LOGR && ((1 << a.logJn) << LOGJ) <= NT;
+}
+// A middle pass before the last one (k_fft_pass_duo): output k of column
+// j = jh Ns + jl is column jl + k Ns of the last pass, row jh.
+FC2_HD bool middle_direct(const PassArgs& a, int LOGR, int LOGJ) {
+    return !a.last && a.logNs + LOGR + a.logRn == a.logM && a.logNs >= a.logJn && a.logNs >= LOGJ;
+}
+// k_fft_first10 before a last pass of radix 2^9 in 16-column tiles (2^19 points).
+FC2_HD bool first10_direct(const PassArgs& a) { return a.logRn == 9 && a.logJn == 4 && a.logM == 19; }
+
 // Last pass: mode m of grid g goes to its place in the spectra.  Grid
 // g < npk (packed) stores F(sh + j) at [2g][j] and F(-(sh + j)) at [2g + 1][j];
 // any other grid stores F(j - hN) at [npk + g][j].
@@ -559,7 +575,7 @@ FC2_D void store_tile_blocked(cpx<T>* __restrict__ gout, const cpx<T>* s, SIdx s
     const int LOGJn = a.logJn, Jn = 1 << a.logJn;
     const int logBlk = a.logRn + a.logJn;
     const int logSn = a.logM - a.logRn;
-    if (logNs == 0 && LOGR <= logSn && LOGJn <= LOGR && (Jn << LOGJ) <= NT) {
+    if (one_stride(a, LOGR, LOGJ, NT)) {
         const int kl = tid & (Jn - 1);
         const int jj = (tid >> LOGJn) & (J - 1);
         const int kb0 = tid >> (LOGJn + LOGJ);
@@ -1618,11 +1634,10 @@ __global__ void __launch_bounds__(DUO_NT, 1) k_fft_pass_duo(const cpx<float>* __
     const int tile0 = blockIdx.x * 2 + grp, tstep = 2 * (int)gridDim.x;
     if (!FIRST && gt == 0 && tile0 < ntiles) issue(tile0);
     const int logNs = a.logNs, nsg_mask = (1 << logNs) - 1, lts = a.logM - logNs - LOGR;
-    const bool same_radix = logNs == 0 && a.logM - a.logRn == LOGR;
-    // a middle pass before the last one: output k of column j = jh Ns + jl is
-    // column jl + k Ns of the last pass, row jh -- contiguous along jl, so the
-    // lanes' runs of columns go straight from registers
-    const bool mid = !a.last && logNs + LOGR + a.logRn == a.logM && logNs >= a.logJn && logNs >= LOGJ;
+    const bool same_radix = two_pass(a, LOGR);
+    // a middle pass before the last one stores contiguously along jl, so the lanes'
+    // runs of columns go straight from registers
+    const bool mid = middle_direct(a, LOGR, LOGJ);
     int it = 0;
     for (int tile = tile0; tile < ntiles; tile += tstep, ++it) {
         const int gl = tile / tiles_x, g = a.g0 + gl, bx = tile - gl * tiles_x, j0 = bx * J;
@@ -1867,8 +1882,7 @@ __global__ void __launch_bounds__(D10_NG * D10_GT, 1) k_fft_first10(const cpx<fl
         return rows > R ? R : rows;
     };
     const int tstep = D10_NG * (int)gridDim.x;
-    // the next pass is the last one, of radix 2^9 in 16-column tiles (2^19 points)
-    const bool direct13 = a.logRn == 9 && a.logJn == 4 && a.logM == LOGR + 9;
+    const bool direct13 = first10_direct(a);
     for (int tile = blockIdx.x * D10_NG + grp; tile < ntiles; tile += tstep) {
         const int gl = tile / tiles_x, g = a.g0 + gl, j0 = (tile - gl * tiles_x) * J;
         const cpx<T>* gin = in + (int64_t)g * M;
@@ -2069,25 +2083,43 @@ static std::vector<int> balanced_plan(int logM, bool fp64) {
 }
 
 // ------------------------------------------------------------ pass kernels
-// Which kernel runs a pass of radix 2^logR (as run_radix chooses), its tile
-// (2^loge elements, 2^logj columns) and threads.
-enum PassKernel { PK_SINGLE = 0, PK_R16 = 1, PK_R64 = 2, PK_BULK = 3, PK_R32 = 4 };
+// Which kernel runs a pass of radix 2^logR, its tile (2^loge elements, 2^logj
+// columns) and the threads that store a tile.  run_radix launches and the host
+// replay follows what pass_shape says.
+enum PassKernel {
+    PK_SINGLE = 0,   // k_fft_pass, the whole transform
+    PK_R16 = 1,      // k_fft_pass
+    PK_R64 = 2,      // k_fft_pass64
+    PK_BULK = 3,     // k_fft_pass_tma
+    PK_R32 = 4,      // k_fft_pass32
+    PK_DUO = 5,      // k_fft_pass_duo
+    PK_FIRST10 = 6,  // k_fft_first10
+    PK_DOUBLE = 7    // k_fft_pass_d (k_fft_pass, the same tiles, where tables are left out)
+};
 struct PassShape {
     int kind, loge, logj, nt;
 };
-static PassShape pass_shape(int logM, bool fp64, int family, int logR) {
+static PassShape pass_shape(int logM, bool fp64, int family, int logR, bool first) {
     if (logR == logM) {
         const int nt = (1 << logR) / 16 < 32 ? 32 : (1 << logR) / 16;
         return PassShape{PK_SINGLE, logR, 0, nt};
     }
-    if (!fp64 && family == FFT_R64 && logR >= 10 && logR <= 12)
+    if (fp64) {
+        const int loge = FftCfg<double>::LOGE;
+        return PassShape{PK_DOUBLE, loge, loge - logR, FftCfg<double>::NT};
+    }
+    if (family == FFT_R64 && logR == 10 && first)
+        return PassShape{PK_FIRST10, PT_LOGE, D10_LOGJ, D10_GT};
+    if (family == FFT_R64 && logR >= 10 && logR <= 12)
         return PassShape{PK_R64, P64_LOGE, P64_LOGE - logR, P64_NT};
-    if (!fp64 && r32_pass(family, logR))
+    if (r32_pass(family, logR))
         return PassShape{PK_R32, P64_LOGE, P64_LOGE - logR, P32_NT};
-    if (!fp64 && family != FFT_R16 && logR >= 8 && logR <= 12)
-        return PassShape{PK_BULK, PT_LOGE, PT_LOGE - logR, logR <= 9 ? DUO_GT : PT_NT};
-    const int loge = fp64 ? FftCfg<double>::LOGE : FftCfg<float>::LOGE;
-    return PassShape{PK_R16, loge, loge - logR, fp64 ? FftCfg<double>::NT : FftCfg<float>::NT};
+    if (family != FFT_R16 && (logR == 8 || logR == 9))
+        return PassShape{PK_DUO, PT_LOGE, PT_LOGE - logR, DUO_GT};
+    if (family != FFT_R16 && logR >= 10 && logR <= 12)
+        return PassShape{PK_BULK, PT_LOGE, PT_LOGE - logR, PT_NT};
+    const int loge = FftCfg<float>::LOGE;
+    return PassShape{PK_R16, loge, loge - logR, FftCfg<float>::NT};
 }
 
 // What the pass kernels assume of a plan (radices rs, first pass first):
@@ -2107,10 +2139,10 @@ static bool fft_plan_valid(int logM, bool fp64, int family, const std::vector<in
     if (rs.size() == 1) return logM >= 9 && logM <= maxr;
     for (size_t i = 0; i < rs.size(); ++i) {
         if (rs[i] < 5 || rs[i] > maxr) return false;
-        const PassShape sh = pass_shape(logM, fp64, family, rs[i]);
+        const PassShape sh = pass_shape(logM, fp64, family, rs[i], i == 0);
         if (sh.logj < 0 || logM - rs[i] < sh.logj) return false;
         if (i + 1 < rs.size()) {
-            const PassShape nx = pass_shape(logM, fp64, family, rs[i + 1]);
+            const PassShape nx = pass_shape(logM, fp64, family, rs[i + 1], false);
             if (nx.logj > rs[i]) return false;
         }
     }
@@ -2303,10 +2335,10 @@ cudaError_t set_fft_choice(fc2_plan_s* p, const FftChoice& c, cudaStream_t s) {
     return init_twiddles(p, s);
 }
 
-// Tile width (columns) of the pass with radix 2^logR.
+// Tile width (columns) of a later pass with radix 2^logR.
 template <typename T>
 static int logj_of(const fc2_plan_s* p, int logR) {
-    return pass_shape(p->logM, sizeof(T) == 8, p->fft_family, logR).logj;
+    return pass_shape(p->logM, sizeof(T) == 8, p->fft_family, logR, false).logj;
 }
 
 
@@ -2479,22 +2511,22 @@ static cudaError_t run_pass_tma(fc2_plan_s* p, const void* in, void* out, const 
 template <typename T, int LOGR>
 static cudaError_t run_radix(fc2_plan_s* p, const void* in, void* out, const PassArgs& a,
                              cudaStream_t s) {
-    if constexpr (sizeof(T) == 4 && LOGR >= 10 && LOGR <= 12) {
-        if (LOGR != p->logM && p->fft_family == FFT_R64) {
-            if (LOGR == 10 && a.first) return run_first10(p, in, out, a, s);
-            return run_pass64<64, LOGR>(p, in, out, a, s);
-        }
+    constexpr bool f32 = sizeof(T) == 4;
+    const int kind = pass_shape(p->logM, !f32, p->fft_family, LOGR, a.first != 0).kind;
+    if constexpr (f32 && LOGR == 10) {
+        if (kind == PK_FIRST10) return run_first10(p, in, out, a, s);
     }
-    if constexpr (sizeof(T) == 4 && (LOGR == 9 || LOGR == 10)) {
-        if (LOGR != p->logM && r32_pass(p->fft_family, LOGR)) return run_pass64<32, LOGR>(p, in, out, a, s);
+    if constexpr (f32 && LOGR >= 10 && LOGR <= 12) {
+        if (kind == PK_R64) return run_pass64<64, LOGR>(p, in, out, a, s);
+        if (kind == PK_BULK) return run_pass_tma<LOGR>(p, in, out, a, s);
     }
-    if constexpr (sizeof(T) == 4 && LOGR >= 8 && LOGR <= 12) {
-        if (LOGR != p->logM && p->fft_family != FFT_R16) {
-            if constexpr (LOGR <= 9) return run_pass_duo<LOGR>(p, in, out, a, s);
-            else return run_pass_tma<LOGR>(p, in, out, a, s);
-        }
+    if constexpr (f32 && (LOGR == 9 || LOGR == 10)) {
+        if (kind == PK_R32) return run_pass64<32, LOGR>(p, in, out, a, s);
     }
-    if (LOGR == p->logM) {
+    if constexpr (f32 && (LOGR == 8 || LOGR == 9)) {
+        if (kind == PK_DUO) return run_pass_duo<LOGR>(p, in, out, a, s);
+    }
+    if (kind == PK_SINGLE) {
         constexpr int NT = (1 << LOGR) / 16 < 32 ? 32 : (1 << LOGR) / 16;
         if constexpr ((1 << LOGR) % (16 * NT) == 0 || (1 << LOGR) >= 16 * NT)
             return run_pass<T, LOGR, 0, NT>(p, in, out, a, s);
@@ -2508,7 +2540,7 @@ static cudaError_t run_radix(fc2_plan_s* p, const void* in, void* out, const Pas
     // harmonics from 6.5 to 5.2 ms).
     // A double call whose tables did not fit (table_room) runs k_fft_pass, which
     // forms the twiddles.
-    if constexpr (sizeof(T) == 8 && LOGJ >= 0) {
+    if constexpr (!f32 && LOGJ >= 0) {
         if (p->fused_fft) return run_pass_d<LOGR, true>(p, in, out, a, s);
         if (a.first || p->d_twpass) return run_pass_d<LOGR, false>(p, in, out, a, s);
     }
@@ -2575,20 +2607,51 @@ cudaError_t launch_fft(fc2_plan_s* p, cudaStream_t s) {
 
 // ------------------------------------------------ host replay of a plan's indices
 // Every global and shared-memory index the pass kernels form for the plan's
-// tiles, replayed on the host with the kernels' own index functions: loads of
-// a pass's input, the stores toward the next pass on each kernel's store path
-// (rows of a same-radix or two-pass plan, the one-stride fast path, the
-// general blocked layout), the shared tile slots read by those stores, and the
-// inter-pass twiddle exponents.  Returns 0 when all of them are in range for
-// the tiles of every pass (all tiles up to 64 per pass, else the first and
-// last 16 and 32 spread between them -- the index functions are monotone
+// tiles, replayed on the host with the kernels' own index functions and route
+// predicates: loads of a pass's input, the stores toward the next pass on the
+// route its kernel takes, the shared tile slots read by those stores, the
+// inter-pass twiddle exponents and the indices into the double passes' tables.
+// Every store must go where the next pass finds that output, and when all tiles
+// are replayed every element must be stored once.  Returns 0 when all of that
+// holds for the tiles of every pass (all tiles up to 64 per pass, else the first
+// and last 16 and 32 spread between them -- the index functions are monotone
 // pieces in the tile number), else 100 * (pass + 1) + the failing check;
 // info[0..3] = pass, check, tile, index.
+enum StoreRoute { ROUTE_NONE = 0, ROUTE_ROWCOL = 1, ROUTE_STRIDE = 2, ROUTE_BLOCKED = 3, ROUTE_DIRECT = 4 };
+static int store_route(const PassShape& sh, const PassArgs& a, int LOGR) {
+    if (a.last) return ROUTE_NONE;
+    switch (sh.kind) {
+        case PK_FIRST10:
+            if (first10_direct(a)) return ROUTE_DIRECT;
+            break;
+        case PK_DUO:
+            if (!a.first && middle_direct(a, LOGR, sh.logj)) return ROUTE_DIRECT;
+            if (two_pass(a, LOGR)) return ROUTE_ROWCOL;
+            break;
+        case PK_R16:
+        case PK_DOUBLE:  // never store_tile_blocked
+            return two_pass(a, LOGR) ? ROUTE_ROWCOL : ROUTE_BLOCKED;
+        default:
+            if (two_pass(a, LOGR)) return ROUTE_ROWCOL;
+    }
+    return one_stride(a, LOGR, sh.logj, sh.nt) ? ROUTE_STRIDE : ROUTE_BLOCKED;
+}
+// The arguments of pass pi of a plan as fft_impl makes them (index part).
+static PassArgs pass_args(int logM, bool fp64, int family, const std::vector<int>& rs, int pi) {
+    PassArgs a{};
+    a.logM = logM;
+    for (int i = 0; i < pi; ++i) a.logNs += rs[i];
+    a.first = pi == 0;
+    a.last = pi + 1 == (int)rs.size();
+    a.logRn = a.last ? 0 : rs[pi + 1];
+    a.logJn = a.last ? 0 : pass_shape(logM, fp64, family, a.logRn, false).logj;
+    return a;
+}
+
 static int replay_plan(int logM, bool fp64, int family, const std::vector<int>& rs,
                        int64_t* info) {
     const int64_t M = 1ll << logM;
     const int P = (int)rs.size();
-    int logNs = 0;
     auto fail = [&](int pi, int check, int64_t tile, int64_t idx) {
         if (info) { info[0] = pi; info[1] = check; info[2] = tile; info[3] = idx; }
         return 100 * (pi + 1) + check;
@@ -2596,16 +2659,14 @@ static int replay_plan(int logM, bool fp64, int family, const std::vector<int>& 
     for (int pi = 0; pi < P; ++pi) {
         const int LOGR = rs[pi];
         const int64_t R = 1ll << LOGR, S = M >> LOGR;
-        PassShape sh = pass_shape(logM, fp64, family, LOGR);
-        // k_fft_first10: 8-column tiles, direct stores for two-pass plans
-        const bool first10 = sh.kind == PK_R64 && LOGR == 10 && pi == 0;
-        if (first10) sh = PassShape{PK_R64, PT_LOGE, D10_LOGJ, DUO_GT};
+        const PassShape sh = pass_shape(logM, fp64, family, LOGR, pi == 0);
+        const PassArgs a = pass_args(logM, fp64, family, rs, pi);
+        const int route = store_route(sh, a, LOGR);
         const int LOGJ = sh.logj, J = 1 << LOGJ;
         const int64_t E = R << LOGJ;
         const bool first = pi == 0, last = pi == P - 1;
-        const int logRn = last ? 0 : rs[pi + 1];
-        const int LOGJn = last ? 0 : pass_shape(logM, fp64, family, logRn).logj;
-        const int logBlk = logRn + LOGJn, logSn = logM - logRn;
+        const int logNs = a.logNs, LOGJn = a.logJn;
+        const int logBlk = a.logRn + LOGJn, logSn = logM - a.logRn;
         const int64_t tiles = S >> LOGJ;
         if (tiles < 1) return fail(pi, 1, 0, S);
         std::vector<int64_t> pick;
@@ -2616,9 +2677,19 @@ static int replay_plan(int logM, bool fp64, int family, const std::vector<int>& 
             for (int64_t t = 16; t < tiles - 16; t += (tiles - 32) / 32 + 1) pick.push_back(t);
             for (int64_t t = tiles - 16; t < tiles; ++t) pick.push_back(t);
         }
-        const bool same_radix = (logNs == 0 && logM - logRn == LOGR);
+        std::vector<uint8_t> stored(!last && tiles <= 64 ? (size_t)M : 0, 0);
+        // a store of output kr of the tile's column jj at gi
+        auto store = [&](int64_t bx, int64_t kr, int64_t jj, int64_t gi) {
+            if (kr < 0 || kr >= R || jj < 0 || jj >= J) return fail(pi, 7, bx, kr * J + jj);
+            if (gi < 0 || gi >= M) return fail(pi, 8, bx, gi);
+            if (gi != blocked_pos(stockham_out((bx << LOGJ) + jj, (int)kr, logNs, LOGR), logSn, LOGJn, logBlk))
+                return fail(pi, 9, bx, gi);
+            if (!stored.empty() && stored[gi]++) return fail(pi, 11, bx, gi);
+            return 0;
+        };
         for (int64_t bx : pick) {
             const int64_t j0 = bx << LOGJ;
+            int rc = 0;
             // loads: the first pass reads rows r < R of columns j0 .. j0 + J - 1;
             // later passes read one contiguous tile of the blocked layout
             const int64_t ld_max = first ? j0 + (J - 1) + (R - 1) * S : bx * E + E - 1;
@@ -2633,87 +2704,93 @@ static int replay_plan(int logM, bool fp64, int family, const std::vector<int>& 
                     qmax = std::max<int64_t>(((RB - 1) * jmax) << lts, ((7 * RB) * jmax) << lts);
                     if (QA > 8)
                         qmax = std::max<int64_t>(qmax, ((8 * RB * ((QA / 8) - 1)) * jmax) << lts);
-                } else if (sh.kind == PK_BULK && bulk_stage1_bits(LOGR) == 5) {
-                    // radix-32 stage 1: t0 up to (R/16 - 1) jm, steps (R/32) jm x 1, 4, 16
-                    qmax = std::max<int64_t>(((R / 16 - 1) * jmax) << lts, ((R / 32) * 16 * jmax) << lts);
-                } else if (fp64) {
-                    // k_fft_pass_d (batches): level 1 of each stage reaches (Q / 2) idx, idx < P / Q,
-                    // P <= D R, in a table of M / 2 entries
-                    for (int done = 0; done < LOGR; done += stage_bits(LOGR, done)) {
-                        const int qb = stage_bits(LOGR, done), logP = logNs + done + qb;
-                        const int64_t idx = jmax + (((1ll << done) - 1) << logNs);
-                        qmax = std::max<int64_t>(qmax, (idx << (qb - 1)) << (logM - logP));
-                        for (int l = 2; l <= qb; ++l)
-                            qmax = std::max<int64_t>(
-                                qmax, ((idx << (qb - l)) + (((1ll << (l - 2)) - 1) << (logP - l)))
-                                          << (logM - logP));
-                    }
-                    if (qmax >= M / 2) return fail(pi, 3, bx, qmax);
-                    const int Q1 = 1 << stage_bits(LOGR, 0);  // k_fft_pass
-                    qmax = std::max<int64_t>(((R / Q1 - 1) * jmax) << lts, ((R / Q1) * jmax) << lts);
+                } else if (sh.kind == PK_DUO && bulk_stage1_bits(LOGR) == 5) {
+                    // radix-32 stage 1: t0 up to (R/32 - 1) jm, steps (R/32) jm x 1, 2, 3, 4, 8, 12, 16
+                    qmax = std::max<int64_t>(((R / 32 - 1) * jmax) << lts, ((R / 32) * 16 * jmax) << lts);
                 } else {
+                    // k_fft_pass, and the plans' tables of double passes, formed the same way
                     const int Q1 = 1 << stage_bits(LOGR, 0);
                     qmax = std::max<int64_t>(((R / Q1 - 1) * jmax) << lts, ((R / Q1) * jmax) << lts);
                 }
                 if (qmax >= M) return fail(pi, 3, bx, qmax);
             }
-            if (last) continue;  // the last pass's mode stores are range-checked
-            if ((sh.kind == PK_R64 || sh.kind == PK_R32 || sh.kind == PK_BULK) && same_radix) {
-                for (int64_t kr = 0; kr < R; ++kr)
-                    for (int jj = 0; jj < J; ++jj) {
-                        const int64_t gi = rowcol_pos((int)kr, j0 + jj, LOGJn, logBlk);
-                        if (gi < 0 || gi >= M) return fail(pi, 4, bx, gi);
-                    }
-                continue;
+            if (sh.kind == PK_DOUBLE) {
+                // k_fft_pass_d's fused form: level 1 of each stage reaches (Q / 2) idx,
+                // idx < P / Q, P <= D R, in a table of M / 2 entries
+                const int64_t jmax = (1ll << logNs) - 1;
+                int64_t qmax = 0;
+                for (int done = 0; done < LOGR; done += stage_bits(LOGR, done)) {
+                    const int qb = stage_bits(LOGR, done), logP = logNs + done + qb;
+                    const int64_t idx = jmax + (((1ll << done) - 1) << logNs);
+                    qmax = std::max<int64_t>(qmax, (idx << (qb - 1)) << (logM - logP));
+                    for (int l = 2; l <= qb; ++l)
+                        qmax = std::max<int64_t>(
+                            qmax, ((idx << (qb - l)) + (((1ll << (l - 2)) - 1) << (logP - l)))
+                                      << (logM - logP));
+                }
+                if (qmax >= M / 2) return fail(pi, 12, bx, qmax);
+                // its other form: the tile's entries in the pass's table, which hold the
+                // twiddles of the tile's columns modulo Ns
+                if (!first) {
+                    const int64_t wt = bx & (pass_tw_tiles(logNs, LOGJ) - 1);
+                    const int64_t top = wt * E + (R - 1) * J + (J - 1);
+                    if (top >= pass_tw_entries(logM, LOGR, 1ll << logNs)) return fail(pi, 13, bx, top);
+                    for (int jj = 0; jj < J; ++jj)
+                        if (((wt * J + jj) & ((1ll << logNs) - 1)) != ((j0 + jj) & ((1ll << logNs) - 1)))
+                            return fail(pi, 14, bx, jj);
+                }
             }
-            const bool fast = (sh.kind == PK_R64 || sh.kind == PK_R32 || sh.kind == PK_BULK) &&
-                              logNs == 0 &&
-                              LOGR <= logSn && LOGJn <= LOGR && (((1 << LOGJn) << LOGJ) <= sh.nt);
-            if (fast) {
+            if (sh.kind == PK_FIRST10 && d10_slot((int)R - 1, J - 1) >= D10_TILE) return fail(pi, 6, bx, R);
+            if (last) continue;  // the last pass's mode stores are range-checked
+            if (route == ROUTE_ROWCOL && sh.kind != PK_DUO && sh.kind != PK_R16 && sh.kind != PK_DOUBLE) {
+                // straight from registers
+                for (int64_t kr = 0; kr < R && !rc; ++kr)
+                    for (int jj = 0; jj < J && !rc; ++jj)
+                        rc = store(bx, kr, jj, rowcol_pos((int)kr, j0 + jj, LOGJn, logBlk));
+            } else if (route == ROUTE_DIRECT && sh.kind == PK_FIRST10) {
+                for (int t = 0; t < D10_GT && !rc; ++t) {
+                    const int pp = t & 15, jj = t >> 4;
+                    for (int k = 0; k < 64 && !rc; ++k)
+                        rc = store(bx, 16 * k + pp, jj, ((j0 + jj) << 4) + pp + (k << 13));
+                }
+            } else if (route == ROUTE_DIRECT) {
+                for (int64_t kr = 0; kr < R && !rc; ++kr)
+                    for (int jj = 0; jj < J && !rc; ++jj) {
+                        const int64_t jl = (j0 + jj) & ((1ll << logNs) - 1), jh = (j0 + jj) >> logNs;
+                        rc = store(bx, kr, jj,
+                                   (((jl >> LOGJn) + (kr << (logNs - LOGJn))) << logBlk) + (jh << LOGJn) +
+                                       (jl & ((1 << LOGJn) - 1)));
+                    }
+            } else if (route == ROUTE_STRIDE) {
                 const int Jn = 1 << LOGJn, NT = sh.nt;
                 const int dkb = NT >> (LOGJn + LOGJ);
-                for (int tid = 0; tid < NT; ++tid) {
+                for (int tid = 0; tid < NT && !rc; ++tid) {
                     const int kl = tid & (Jn - 1);
                     const int jj = (tid >> LOGJn) & (J - 1);
                     const int kb0 = tid >> (LOGJn + LOGJ);
                     const int64_t i0 = (j0 + jj) << LOGR;
                     const int64_t jb = i0 & ((1ll << logSn) - 1), rn = i0 >> logSn;
                     const int e0 = (kb0 << (LOGJn + LOGJ)) + (kl << LOGJ) + jj;
-                    for (int64_t it = 0; it < E / NT; ++it) {
+                    for (int64_t it = 0; it < E / NT && !rc; ++it) {
                         const int64_t gi = (((jb >> LOGJn) + kb0 + it * dkb) << logBlk) +
                                            (rn << LOGJn) + kl;
-                        const int64_t se = e0 + it * NT;
-                        if (gi < 0 || gi >= M) return fail(pi, 5, bx, gi);
+                        const int64_t se = e0 + it * NT;  // k J + jj
                         if (se < 0 || se >= E) return fail(pi, 6, bx, se);
+                        rc = store(bx, se >> LOGJ, se & (J - 1), gi);
                     }
                 }
-                continue;
+            } else {
+                for (int64_t e = 0; e < E && !rc; ++e) {
+                    const TileElem te = tile_elem((int)e, LOGJn, LOGJ);
+                    rc = store(bx, te.k, te.jj,
+                               route == ROUTE_ROWCOL
+                                   ? rowcol_pos(te.k, j0 + te.jj, LOGJn, logBlk)
+                                   : blocked_pos(stockham_out(j0 + te.jj, te.k, logNs, LOGR), logSn,
+                                                 LOGJn, logBlk));
+                }
             }
-            if (sh.kind == PK_BULK && LOGR <= 9 && !first && logNs + LOGR + logRn == logM &&
-                logNs >= LOGJn && logNs >= LOGJ) {  // k_fft_pass_duo's direct middle store
-                for (int64_t kr = 0; kr < R; ++kr)
-                    for (int jj = 0; jj < J; ++jj) {
-                        const int64_t jl = (j0 + jj) & ((1ll << logNs) - 1), jh = (j0 + jj) >> logNs;
-                        const int64_t gi = (((jl >> LOGJn) + (kr << (logNs - LOGJn))) << logBlk) +
-                                           (jh << LOGJn) + (jl & ((1 << LOGJn) - 1));
-                        if (gi < 0 || gi >= M ||
-                            gi != blocked_pos(stockham_out(j0 + jj, (int)kr, logNs, LOGR), logSn, LOGJn,
-                                              logBlk))
-                            return fail(pi, 9, bx, gi);
-                    }
-                continue;
-            }
-            const bool rowcol = sh.kind == PK_R16 && same_radix;
-            for (int64_t e = 0; e < E; ++e) {
-                const TileElem te = tile_elem((int)e, LOGJn, LOGJ);
-                if (te.k >= R || te.jj >= J) return fail(pi, 7, bx, (int64_t)te.k * J + te.jj);
-                const int64_t gi = rowcol ? rowcol_pos(te.k, j0 + te.jj, LOGJn, logBlk)
-                                          : blocked_pos(stockham_out(j0 + te.jj, te.k, logNs, LOGR),
-                                                        logSn, LOGJn, logBlk);
-                if (gi < 0 || gi >= M) return fail(pi, 8, bx, gi);
-            }
+            if (rc) return rc;
         }
-        logNs += LOGR;
     }
     return 0;
 }
@@ -2753,4 +2830,18 @@ extern "C" int fc2_debug_fft_plan_check(int logM, int fp64, int fft_kernel, cons
     const int fam = fc2::fft_family_of(fft_kernel);
     if (validate && !fc2::fft_plan_valid(logM, fp64 != 0, fam, rs)) return 1;
     return fc2::replay_plan(logM, fp64 != 0, fam, rs, info4);
+}
+
+extern "C" int fc2_debug_fft_pass(int logM, int fp64, int fft_kernel, const int* radices, int P,
+                                  int pass, int* out4) {
+    if (!radices || !out4 || P < 1 || P > 8 || pass < 0 || pass >= P || logM < 1 || logM > 40) return -1;
+    const std::vector<int> rs(radices, radices + P);
+    const int fam = fc2::fft_family_of(fft_kernel);
+    if (!fc2::fft_plan_valid(logM, fp64 != 0, fam, rs)) return 1;
+    const fc2::PassShape sh = fc2::pass_shape(logM, fp64 != 0, fam, rs[pass], pass == 0);
+    out4[0] = sh.kind;
+    out4[1] = sh.logj;
+    out4[2] = sh.nt;
+    out4[3] = fc2::store_route(sh, fc2::pass_args(logM, fp64 != 0, fam, rs, pass), rs[pass]);
+    return 0;
 }
