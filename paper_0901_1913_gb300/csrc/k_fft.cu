@@ -460,8 +460,10 @@ FC2_HD bool one_stride(const PassArgs& a, int LOGR, int LOGJ, int NT) {
 FC2_HD bool middle_direct(const PassArgs& a, int LOGR, int LOGJ) {
     return !a.last && a.logNs + LOGR + a.logRn == a.logM && a.logNs >= a.logJn && a.logNs >= LOGJ;
 }
-// k_fft_first10 before a last pass of radix 2^9 in 16-column tiles (2^19 points).
-FC2_HD bool first10_direct(const PassArgs& a) { return a.logRn == 9 && a.logJn == 4 && a.logM == 19; }
+// k_fft_first10 before a last pass of 16-column tiles: the 16 rows of a half-warp
+// are one 128-byte line of its layout (24 grids of 2^20: both passes 264 us with
+// the results staged, 249 so; 207 and 198 with one row in a thousand occupied).
+FC2_HD bool first10_direct(const PassArgs& a) { return two_pass(a, 10) && a.logJn == 4; }
 
 // Last pass: mode m of grid g goes to its place in the spectra.  Grid
 // g < npk (packed) stores F(sh + j) at [2g][j] and F(-(sh + j)) at [2g + 1][j];
@@ -1882,7 +1884,7 @@ __global__ void __launch_bounds__(D10_NG * D10_GT, 1) k_fft_first10(const cpx<fl
         return rows > R ? R : rows;
     };
     const int tstep = D10_NG * (int)gridDim.x;
-    const bool direct13 = first10_direct(a);
+    const bool direct = first10_direct(a);
     for (int tile = blockIdx.x * D10_NG + grp; tile < ntiles; tile += tstep) {
         const int gl = tile / tiles_x, g = a.g0 + gl, j0 = (tile - gl * tiles_x) * J;
         const cpx<T>* gin = in + (int64_t)g * M;
@@ -1933,9 +1935,11 @@ __global__ void __launch_bounds__(D10_NG * D10_GT, 1) k_fft_first10(const cpx<fl
 #pragma unroll
         for (int k = 1; k < 64; ++k) v[k] = mul(v[k], st[(k - 1) * QA + pp]);
         SmallDFT<T, 64>::run(v);
-        if (direct13) {  // rows 16 k + pp: block k, row pp of it
+        if (direct) {  // rows 16 k + pp: block k, row pp of it
+            cpx<T>* dst = gout + ((int64_t)(j0 + jj) << 4) + pp;
+            const int64_t blk = 1ll << (a.logRn + 4);
 #pragma unroll
-            for (int k = 0; k < 64; ++k) gout[((j0 + jj) << 4) + pp + (k << 13)] = v[k];
+            for (int k = 0; k < 64; ++k) dst[k * blk] = v[k];
         } else {
             d10_sync(grp);
 #pragma unroll
@@ -2751,7 +2755,7 @@ static int replay_plan(int logM, bool fp64, int family, const std::vector<int>& 
                 for (int t = 0; t < D10_GT && !rc; ++t) {
                     const int pp = t & 15, jj = t >> 4;
                     for (int k = 0; k < 64 && !rc; ++k)
-                        rc = store(bx, 16 * k + pp, jj, ((j0 + jj) << 4) + pp + (k << 13));
+                        rc = store(bx, 16 * k + pp, jj, ((j0 + jj) << 4) + pp + ((int64_t)k << (a.logRn + 4)));
                 }
             } else if (route == ROUTE_DIRECT) {
                 for (int64_t kr = 0; kr < R && !rc; ++kr)

@@ -34,7 +34,7 @@ def info(lib, rs, p, fp64=0, kernel=DEFAULT):
 def test_first_pass_of_radix_2_10(lib):
     # three groups of 128 threads, each with a tile of 8 columns
     assert info(lib, [10, 9], 0) == (FIRST10, 3, 128, DIRECT)      # 2^19 points
-    assert info(lib, [10, 10], 0)[:3] == (FIRST10, 3, 128)
+    assert info(lib, [10, 10], 0) == (FIRST10, 3, 128, DIRECT)     # 2^20: the same layout
     assert info(lib, [10, 9, 9], 0) == (FIRST10, 3, 128, STRIDE)   # next tile: 16 columns
     # a next tile of 32 columns: 32 x 8 elements are more than a group's threads
     assert info(lib, [10, 8], 0) == (FIRST10, 3, 128, BLOCKED)
