@@ -16,11 +16,11 @@
 // of that (2H)-square system gives every H' at once (Sec. 1).  Everything is
 // normalised by W and sqrt(W chi2_poly), so Delta chi^2' lies in [0, 1].
 //
-// The gridded pass solves one trial frequency per thread in double and flags
-// bins whose estimated error is too large; those, and the records, are
-// recomputed from exact double sums over the samples (the Q and P sums of the
-// double fix-up tier plus the trend sums T), one warp per bin: lane l holds
-// harmonic column l + 1.
+// The gridded pass solves one trial frequency per thread in double (per warp on
+// short trial grids) and flags bins whose estimated error is too large; those,
+// and the records, are recomputed from exact double sums over the samples (the Q
+// and P sums of the double fix-up tier plus the trend sums T), one warp per bin:
+// lane l holds harmonic column l + 1.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -48,13 +48,15 @@ struct JointParams {
 // Harmonic-column solve of the projected system for one bin.  S holds the
 // normalised Q (qr/qi, k = 0..2H) and P (pr/pi, k = 1..H) sums, T the
 // normalised trend sums T_{p,h} at [(p - 1) H + h - 1] (re, im).  Every lane
-// returns out[H' - 1] = Delta chi^2'_{H'}; with coef != nullptr, coef[0..2Hc)
+// returns out[H' - 1] = Delta chi^2'_{H'} and the smallest relative pivot.
+// With COEF, *anorm2 = max over H' <= H of the harmonic coefficient norm
+// |A_H'|^2 (float, for the error estimate); with coef != nullptr, coef[0..2Hc)
 // gets the Hc-harmonic coefficients and poly[0..D] the polynomial ones
 // (normalised units).
-template <int H, int D>
-FC2_D void warp_joint_solve(const Sys<double, H>& S, const double* Tre, const double* Tim,
-                            const JointParams& jp, double* out, double* coef = nullptr,
-                            int Hc = 0, double* poly = nullptr) {
+template <int H, int D, bool COEF>
+FC2_D double warp_joint_solve(const Sys<double, H>& S, const double* Tre, const double* Tim,
+                              const JointParams& jp, double* out, double* anorm2,
+                              double* coef = nullptr, int Hc = 0, double* poly = nullptr) {
     constexpr int m = 2 * H;
     static_assert(m <= 32, "one column per lane");
     constexpr unsigned FULL = 0xffffffffu;
@@ -99,6 +101,7 @@ FC2_D void warp_joint_solve(const Sys<double, H>& S, const double* Tre, const do
     // right-looking Cholesky, lane l holding row l
     double Lr[m], z[m], dinv[m];
     double acc = 0.0;
+    float dmin = 1.0f;
 #pragma unroll
     for (int k = 0; k < m; ++k) {
         const double dk = __shfl_sync(FULL, a[k], k);
@@ -117,8 +120,31 @@ FC2_D void warp_joint_solve(const Sys<double, H>& S, const double* Tre, const do
             if (j <= l) a[j] = fma(-Llk, Ljk, a[j]);
         }
         b = fma(-Llk, zk, b);
+        const float rc = allk > 0.0 ? fmaxf((float)dk / (float)allk, 0.0f) : 0.0f;
+        dmin = fminf(dmin, rc);
         acc = fma(zk, zk, acc);
         if ((k & 1) == 1) out[k >> 1] = acc;
+    }
+    if constexpr (COEF) {
+        float amax = 0.0f;
+#pragma unroll
+        for (int hp = 1; hp <= H; ++hp) {
+            const int mp = 2 * hp;
+            float mine = 0.0f, nrm = 0.0f;
+#pragma unroll
+            for (int k = m - 1; k >= 0; --k) {
+                if (k < mp) {
+                    float t = (l > k && l < mp) ? (float)Lr[k] * mine : 0.0f;
+#pragma unroll
+                    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(FULL, t, o);
+                    const float A = ((float)z[k] - t) * (float)dinv[k];
+                    if (l == k) mine = A;
+                    nrm = fmaf(A, A, nrm);
+                }
+            }
+            amax = fmaxf(amax, nrm);
+        }
+        *anorm2 = (double)amax;
     }
     if (coef) {
         const int mp = 2 * Hc;
@@ -153,6 +179,7 @@ FC2_D void warp_joint_solve(const Sys<double, H>& S, const double* Tre, const do
             poly[p] = v / jp.LG[p * 4 + p];
         }
     }
+    return (double)dmin;
 }
 
 // ---------------------------------------------------------- gridded pass
@@ -296,6 +323,67 @@ __global__ void __launch_bounds__(128) k_assemble_joint(const cpx<TS>* __restric
     }
 }
 
+// The same with one warp per bin (lane l holds column l + 1), for trial grids so
+// short that warps of 32 bins leave SM sub-partitions without work: a thread's
+// chain of some 300 (H = 3) to 3000 (H = 8) double operations takes as long for
+// one bin as for 32.  One, two and three warps a sub-partition (608 bins each)
+// against the form above, float spectra:
+//   H = 3, D = 3   22, 32, 44 us against 27      H = 6, D = 2   32, 48, 67 us against 59
+//   H = 4, D = 2   24, 34, 47     against 34     H = 7, D = 3    -,  -, 85     against 89
+//   H = 5, D = 2   28, 40, 56     against 44     H = 8, D = 2   44, 63, 89     against 103
+// (2400 bins at H = 8: 151 to 104; one and two harmonics: as fast by threads).
+constexpr int64_t JOINT_WAVE = 4 * 152;
+inline bool joint_by_warps(int64_t N, int H) {
+    return N <= JOINT_WAVE * (H < 3 ? 0 : H < 4 ? 1 : H < 7 ? 2 : 3);
+}
+
+template <typename TS, int H, int D>
+__global__ void __launch_bounds__(128) k_assemble_joint_warp(const cpx<TS>* __restrict__ spec,
+                                                             const TS* __restrict__ dec,
+                                                             double* __restrict__ dchi2,
+                                                             JointParams jp, double dmin_exact,
+                                                             int32_t* __restrict__ list,
+                                                             int32_t* __restrict__ list_count,
+                                                             int64_t cap) {
+    const int64_t wpb = blockDim.x >> 5;
+    for (int64_t j = (int64_t)blockIdx.x * wpb + (threadIdx.x >> 5); j < jp.N;
+         j += (int64_t)gridDim.x * wpb) {
+        const double d = (double)dec[j];
+        const double dq = d * jp.sq, dp = d * jp.jsp;
+        Sys<double, H> S;
+        S.qr[0] = 1.0; S.qi[0] = 0.0; S.pr[0] = 0.0; S.pi[0] = 0.0;
+#pragma unroll
+        for (int k = 1; k <= 2 * H; ++k) {
+            const cpx<TS> v = spec[(int64_t)(k - 1) * jp.N + j];
+            S.qr[k] = (double)v.x * dq;
+            S.qi[k] = (double)v.y * dq;
+        }
+#pragma unroll
+        for (int k = 1; k <= H; ++k) {
+            const cpx<TS> v = spec[(int64_t)(2 * H + k - 1) * jp.N + j];
+            S.pr[k] = (double)v.x * dp;
+            S.pi[k] = (double)v.y * dp;
+        }
+        double Tre[D * H], Tim[D * H];
+#pragma unroll
+        for (int q = 0; q < D * H; ++q) {
+            const cpx<TS> v = spec[(int64_t)(3 * H + q) * jp.N + j];
+            Tre[q] = (double)v.x * dq;
+            Tim[q] = (double)v.y * dq;
+        }
+        double out[H], an2 = 0.0;
+        const double dmin = warp_joint_solve<H, D, true>(S, Tre, Tim, jp, out, &an2);
+        if ((threadIdx.x & 31) == 0) {
+            if (!(est_err<double>(an2, 2 * H + 1 + D, jp.eps) <= jp.err_fix) || dmin < dmin_exact) {
+                const int32_t pos = atomicAdd(list_count, 1);
+                if (pos < cap) list[pos] = (int32_t)j;
+            }
+#pragma unroll
+            for (int hh = 0; hh < H; ++hh) dchi2[(int64_t)hh * jp.N + j] = out[hh] * jp.chi0;
+        }
+    }
+}
+
 // ------------------------------------------------------ exact trend sums
 // T_{p,k} = sum_i w_i u_i^p e^{2 pi i k f tau_i} (p = 1..D, k = 1..H) in double,
 // u_i = (tau_i - tc) is, for work items (bin, chunk of samples) laid out as the
@@ -415,8 +503,8 @@ __global__ void __launch_bounds__(128) k_exact_joint_dchi2(
     Sys<double, H> S;
     double Tre[D * H], Tim[D * H];
     joint_exact_sys<H, D>(part, part_t, b, nch, scal, sh[w], sht[w], S, Tre, Tim);
-    double out[H];
-    warp_joint_solve<H, D>(S, Tre, Tim, jp, out);
+    double out[H], an2 = 0.0;
+    warp_joint_solve<H, D, false>(S, Tre, Tim, jp, out, &an2);
     if ((threadIdx.x & 31) != 0) return;
     const int64_t j = list[base + b];
 #pragma unroll
@@ -449,8 +537,8 @@ __global__ void __launch_bounds__(128) k_exact_joint_coeffs(
     Sys<double, H> S;
     double Tre[D * H], Tim[D * H];
     joint_exact_sys<H, D>(part, part_t, r, nch, scal, sh[w], sht[w], S, Tre, Tim);
-    double o[H], coef[2 * H], poly[D + 1];
-    warp_joint_solve<H, D>(S, Tre, Tim, jp, o, coef, Hp, poly);
+    double o[H], an2 = 0.0, coef[2 * H], poly[D + 1];
+    warp_joint_solve<H, D, false>(S, Tre, Tim, jp, o, &an2, coef, Hp, poly);
     if ((threadIdx.x & 31) != 0) return;
     const double W = scal[SC_W];
     const double unit = (W > 0.0) ? sqrt(jp.chi0 / W) : 0.0;
@@ -501,6 +589,13 @@ static cudaError_t assemble_joint_impl(fc2_plan_s* p, cudaStream_t s) {
     const double dmin_exact = p->fp64 ? 1e-11 : 1e-7;
 #define FC2_JA(HH, DD)                                                                        \
     if (p->H == HH && p->D == DD) {                                                           \
+        if constexpr (HH >= 3) {                                                              \
+            if (joint_by_warps(p->N, HH)) {                                                   \
+                k_assemble_joint_warp<TS, HH, DD><<<(unsigned)((p->N + 3) / 4), 128, 0, s>>>( \
+                    spec, dec, p->d_dchi2, jp, dmin_exact, list, cnt, p->flag_cap);           \
+                return cudaGetLastError();                                                    \
+            }                                                                                 \
+        }                                                                                     \
         k_assemble_joint<TS, HH, DD><<<blocks, 128, 0, s>>>(spec, dec, p->d_dchi2, jp,        \
                                                             dmin_exact, list, cnt,            \
                                                             p->flag_cap);                     \
