@@ -52,6 +52,12 @@ FC2_D float narrow_est(double v) {
     return copysignf(d2f_trunc(fabs(v)), (float)(__double2hiint(v) >> 31 | 1));
 }
 
+// The larger of two coefficient norms.  A norm beyond float's range (infinity, or
+// NaN where infinities met) counts as infinite: its bin is recomputed.
+FC2_D float larger_norm(float a, float nrm) {
+    return fmaxf(a, nrm == nrm ? nrm : __int_as_float(0x7f800000));
+}
+
 // Factor and solve; out[H'-1] = Delta chi^2'_{H'}.  Returns the minimum
 // relative pivot over all columns (clamped at 0).  With COEF, *anorm2 receives
 // max over H' of |A^{(H')}|^2 (A^{(H')} = the H'-harmonic coefficients, by
@@ -107,7 +113,10 @@ FC2_D TC chol_solve(const Sys<TC, H>& S, TC tau, TC* out, TC* anorm2,
     if constexpr (COEF) {
         // in float also for a double solve: the norm only feeds the error estimate,
         // and its back-substitutions were 20-25% of the double operations
-        // (32 curves, N = 2^18, H = 2..6: 9.4 -> 8.3 ms; 2^20 bins, H = 4: 1086 -> 965 us)
+        // (32 curves, N = 2^18, H = 2..6: 9.4 -> 8.3 ms; 2^20 bins, H = 4: 1086 -> 965 us).
+        // Triangular systems are solved to some m 2^-22 whatever their condition in
+        // practice (1.3e-5 of the norm at most over nearly singular bins of 1..8
+        // harmonics), where the estimate itself is good to a factor.
         float Lf[m][m], zf[m], df[m], amax = 0.f;
 #pragma unroll
         for (int l = 0; l < m; ++l) {
@@ -132,7 +141,7 @@ FC2_D TC chol_solve(const Sys<TC, H>& S, TC tau, TC* out, TC* anorm2,
                     nrm = fmaf(A[l], A[l], nrm);
                 }
             }
-            amax = nrm > amax ? nrm : amax;
+            amax = larger_norm(amax, nrm);
         }
         *anorm2 = (TC)amax;
     }
@@ -215,7 +224,7 @@ FC2_D double warp_chol_solve(const Sys<double, H>& S, double tau, double* out, d
                     nrm = fmaf(A, A, nrm);
                 }
             }
-            amax = fmaxf(amax, nrm);
+            amax = larger_norm(amax, nrm);
         }
         *anorm2 = (double)amax;
     }

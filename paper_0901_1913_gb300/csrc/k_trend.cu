@@ -142,7 +142,7 @@ FC2_D double warp_joint_solve(const Sys<double, H>& S, const double* Tre, const 
                     nrm = fmaf(A, A, nrm);
                 }
             }
-            amax = fmaxf(amax, nrm);
+            amax = larger_norm(amax, nrm);
         }
         *anorm2 = (double)amax;
     }
@@ -314,7 +314,7 @@ __global__ void __launch_bounds__(128) k_assemble_joint(const cpx<TS>* __restric
                 nrm = fmaf(A[k], A[k], nrm);
             }
         }
-        amax = fmaxf(amax, nrm);
+        amax = larger_norm(amax, nrm);
     }
     if (!(est_err<double>((double)amax, 2 * H + 1 + D, jp.eps) <= jp.err_fix) ||
         (double)dmin < dmin_exact) {
