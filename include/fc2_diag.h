@@ -54,6 +54,12 @@ void fc2_debug_counts(fc2_plan p, int64_t* out7);
  * fails. */
 fc2_status fc2_debug_spectra(fc2_plan p, double* re, double* im);
 
+/* The transform passes of a double-precision plan in the fused form that
+ * batches run (fused != 0: other rounding, the same accuracy) or in the plan's
+ * own form again, from the next execute on; for tests of the spectra.
+ * FC2_ERR_INVALID_ARG on NULL or a mixed plan. */
+fc2_status fc2_debug_fused_passes(fc2_plan p, int fused);
+
 /* The time origin T0 the plan measures phases from (Sec. 3b); 0 on NULL. */
 double fc2_debug_t0(fc2_plan p);
 
@@ -183,6 +189,16 @@ fc2_status fc2_debug_phasor(const uint64_t* u, int64_t n, float* out4);
  * point): one double-float table entry e^{2 pi i m / 65536} for the top 16
  * bits, then the same small rotation.  Same arguments and errors. */
 fc2_status fc2_debug_phasor16(const uint64_t* u, int64_t n, float* out4);
+
+/* The trigonometric sums of one entry of a batch as one warp of the exact fix-up
+ * forms them: samples i < n of phases (A_i + j B_i) 2^-64 turns, weights wq
+ * and weighted data wp, H harmonics, padded to a capacity of 4, 6 or 8, by
+ * tier 3 or 4.  out[6 capacity]: re, im of Q_k (k = 1..2 capacity), then of
+ * P_k (k = 1..capacity), zero beyond 2H and H.  Host arrays.  For tests of
+ * their accuracy.  FC2_ERR_INVALID_ARG for bad arguments. */
+fc2_status fc2_debug_batch_sums(const uint64_t* A, const uint64_t* B, const double* wq,
+                                const double* wp, int64_t n, int64_t j, int H, int capacity,
+                                int tier, double* out);
 
 /* Launch configuration of the last fc2_execute_batched call's last chunk
  * (out12): [0] source (0 fixed, 1 tuning table or cache file, 2 tuned in the

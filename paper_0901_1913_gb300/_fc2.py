@@ -164,6 +164,8 @@ def load():
         lib.fc2_debug_last_tier.restype = None
         lib.fc2_debug_fail_alloc.argtypes = [i64]
         lib.fc2_debug_fail_alloc.restype = None
+        lib.fc2_debug_fused_passes.argtypes = [_P, i32]
+        lib.fc2_debug_fused_passes.restype = i32
         lib.fc2_debug_table_memory.argtypes = [i64]
         lib.fc2_debug_table_memory.restype = None
         lib.fc2_debug_alloc_count.argtypes = []
@@ -328,6 +330,10 @@ class Plan:
         im = np.empty(G * self.N)
         _check(load().fc2_debug_spectra(self.h, re.ctypes.data, im.ctypes.data), "spectra")
         return (re + 1j * im).reshape(G, self.N)
+
+    def fused_passes(self, on=True):
+        """A double plan's transform passes in the form batches run (for tests)."""
+        _check(load().fc2_debug_fused_passes(self.h, int(on)), "fc2_debug_fused_passes")
 
     def stage_timing(self, enable=True):
         _check(load().fc2_stage_timing(self.h, int(enable)), "fc2_stage_timing")

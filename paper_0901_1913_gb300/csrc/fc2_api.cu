@@ -839,6 +839,30 @@ fc2_status fc2_debug_fault(fc2_plan p, long long wait_cycles, int drop_tile) {
     return FC2_OK;
 }
 
+/* The transform passes of a double plan in the fused form that batches run
+ * (fused != 0) or in the plan's own, for tests of its spectra. */
+fc2_status fc2_debug_fused_passes(fc2_plan p, int fused) {
+    if (!p || !p->fp64) return FC2_ERR_INVALID_ARG;
+    if (cudaSetDevice(p->device) != cudaSuccess) return FC2_ERR_CUDA;
+    cudaStream_t s = p->stream;
+    int sh;
+    int64_t nlo, nhi;
+    twiddle_split(p->logM, fused != 0, &sh, &nlo, &nhi);
+    void *lo = nullptr, *hi = nullptr;
+    Guard g;
+    g.ok(dalloc(&lo, (size_t)nlo * 16, s)) && g.ok(dalloc(&hi, (size_t)nhi * 16, s));
+    if (g.e != cudaSuccess) {
+        dfree(lo, s); dfree(hi, s);
+        return map_err(g.e);
+    }
+    std::swap(lo, p->d_twlo);
+    std::swap(hi, p->d_twhi);
+    p->fused_fft = fused != 0;
+    dfree(lo, s); dfree(hi, s);
+    g.ok(init_twiddles(p, s)) && g.ok(cudaStreamSynchronize(s));
+    return map_err(g.e);
+}
+
 /* Bins of the last execute that tier `tier` (2 or 3) of the exact fix-up
  * handled; returns how many were copied (at most cap), or -1. */
 int64_t fc2_debug_tier_bins(fc2_plan p, int tier, int64_t* out, int64_t cap) {
@@ -890,6 +914,17 @@ fc2_status fc2_debug_phasor(const uint64_t* u, int64_t n, float* out4) {
 fc2_status fc2_debug_phasor16(const uint64_t* u, int64_t n, float* out4) {
     if (!u || !out4 || n < 1 || n > (1 << 24)) return FC2_ERR_INVALID_ARG;
     return fc2::debug_phasor(u, n, 1, out4) == cudaSuccess ? FC2_OK : FC2_ERR_CUDA;
+}
+
+/* The exact sums of one entry of a batch as one warp forms them (host arrays). */
+fc2_status fc2_debug_batch_sums(const uint64_t* A, const uint64_t* B, const double* wq,
+                                const double* wp, int64_t n, int64_t j, int H, int capacity,
+                                int tier, double* out) {
+    if (!A || !B || !wq || !wp || !out || n < 1 || n > (1 << 24) || j < 0 || H < 1 || H > capacity ||
+        (capacity != 4 && capacity != 6 && capacity != 8) || (tier != 3 && tier != 4))
+        return FC2_ERR_INVALID_ARG;
+    return fc2::debug_batch_sums(A, B, wq, wp, n, j, H, capacity, tier, out) == cudaSuccess ? FC2_OK
+                                                                                           : FC2_ERR_CUDA;
 }
 
 /* Kernels launched by the last fc2_execute_batched call of this process. */

@@ -309,6 +309,8 @@ cudaError_t launch_phase_fx(fc2_plan_s* p, cudaStream_t s);
 // into tab (2 * 512 * 16 bytes).
 cudaError_t launch_init_dftab(void* tab, bool with16, cudaStream_t s);  // with16: also DFTAB_T16's table
 cudaError_t debug_phasor(const uint64_t* u, int64_t n, int table16, float* out4);  // diagnostics
+cudaError_t debug_batch_sums(const uint64_t* A, const uint64_t* B, const double* wq, const double* wp,
+                             int64_t n, int64_t j, int H, int capacity, int tier, double* out);
 
 // k_adjoint.cu: one entry = (curve << 32 | bin) of a curve table
 struct AdjTab {

@@ -2386,4 +2386,61 @@ fc2_status batched_backward(int64_t C, const int64_t* offsets, const double* t, 
     return map_cuda(e);
 }
 
+// The sums of one entry by one warp (diagnostics: their accuracy test).
+template <int HM, int TIER>
+__global__ void k_debug_bx_sums(const uint64_t* __restrict__ A, const uint64_t* __restrict__ B,
+                                const float* __restrict__ wq32, const float* __restrict__ wp32,
+                                const double* __restrict__ wq, const double* __restrict__ wp,
+                                const dfc* __restrict__ dftab, int64_t n, uint64_t ju, int H,
+                                double* __restrict__ out) {
+    __shared__ BxTables<TIER> tb;
+    tb.load(dftab);
+    double tot[6 * HM];
+    bx_sums<HM, TIER>(A, B, wq32, wp32, wq, wp, tb, n, ju, H, 0, n, threadIdx.x & 31, tot);
+    if (threadIdx.x == 0)
+        for (int v = 0; v < 6 * HM; ++v) out[v] = tot[v];
+}
+
+cudaError_t debug_batch_sums(const uint64_t* A, const uint64_t* B, const double* wq, const double* wp,
+                             int64_t n, int64_t j, int H, int capacity, int tier, double* out) {
+    std::vector<float> w32((size_t)4 * n);  // high and low parts of wq, then of wp
+    for (int64_t i = 0; i < n; ++i) {
+        for (int q = 0; q < 2; ++q) {
+            const double w = q ? wp[i] : wq[i];
+            const float hi = (float)w;
+            w32[(2 * q) * n + i] = hi;
+            w32[(2 * q + 1) * n + i] = (float)(w - (double)hi);
+        }
+    }
+    void *dA = nullptr, *dB = nullptr, *dq = nullptr, *dp = nullptr, *d32 = nullptr, *tab = nullptr, *o = nullptr;
+    cudaError_t e = cudaSuccess;
+    auto ok = [&](cudaError_t r) { if (e == cudaSuccess) e = r; };
+    auto up = [&](void** d, const void* h, size_t bytes) {
+        ok(cudaMalloc(d, bytes));
+        if (e == cudaSuccess && h) ok(cudaMemcpy(*d, h, bytes, cudaMemcpyHostToDevice));
+    };
+    up(&dA, A, n * 8); up(&dB, B, n * 8); up(&dq, wq, n * 8); up(&dp, wp, n * 8);
+    up(&d32, w32.data(), w32.size() * 4); up(&tab, nullptr, 2 * 512 * 16); up(&o, nullptr, 6 * BHM * 8);
+    if (e == cudaSuccess) ok(launch_init_dftab(tab, false, 0));
+    if (e == cudaSuccess) {
+        const float* q32 = (const float*)d32;
+        auto run = [&](auto hm, auto t) {
+            k_debug_bx_sums<decltype(hm)::value, decltype(t)::value><<<1, 32>>>(
+                (const uint64_t*)dA, (const uint64_t*)dB, q32, q32 + 2 * n, (const double*)dq,
+                (const double*)dp, (const dfc*)tab, n, (uint64_t)j, H, (double*)o);
+        };
+        auto by_tier = [&](auto hm) {
+            if (tier == 4) run(hm, std::integral_constant<int, 4>{});
+            else run(hm, std::integral_constant<int, 3>{});
+        };
+        if (capacity == 4) by_tier(std::integral_constant<int, 4>{});
+        else if (capacity == 6) by_tier(std::integral_constant<int, 6>{});
+        else by_tier(std::integral_constant<int, BHM>{});
+        ok(cudaGetLastError());
+        ok(cudaMemcpy(out, o, (size_t)6 * capacity * 8, cudaMemcpyDeviceToHost));
+    }
+    for (void* d : {dA, dB, dq, dp, d32, tab, o}) cudaFree(d);
+    return e;
+}
+
 }  // namespace fc2

@@ -2033,7 +2033,7 @@ cudaError_t init_twiddles(fc2_plan_s* p, cudaStream_t s) {
     else
         k_init_tw<float><<<blocks, 256, 0, s>>>((cpx<float>*)p->d_twlo, nlo,
                                                 (cpx<float>*)p->d_twhi, nhi, p->logM, sh);
-    if (p->d_twpass) {
+    if (p->d_twpass && !p->fused_fft) {
         cpx<double>* tab = (cpx<double>*)p->d_twpass;
         for (const auto& ps : p->passes) {
             const int64_t n = pass_tw_entries(p->logM, ps.logR, ps.Ns);
