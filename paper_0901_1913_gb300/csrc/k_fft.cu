@@ -780,11 +780,11 @@ __global__ void k_init_pass_tw(cpx<double>* __restrict__ tab, int logM, int logD
 
 // The pass of k_fft_pass in double: the same tiles, layouts and stages.  FUSED
 // (batches): dit_stage's butterflies with the merged twiddles of the table twf
-// (q < M / 2).  Otherwise (plans) k_fft_pass's operations in its order, results
-// bit-equal, with the inter-pass twiddles from a table (twf, k_init_pass_tw: four
+// (q < M / 2).  Otherwise (plans) k_fft_pass's operations in its order, with its
+// results, the inter-pass twiddles from a table (twf, k_init_pass_tw: four
 // operations per element where forming them took eleven) and the zero rows and
 // unwanted modes skipped (12 grids of 2^21: 3.71 -> 3.11 ms); twst: the stage
-// twiddles.
+// twiddles.  Where the tables are left out for want of memory k_fft_pass runs.
 template <int LOGR, int LOGJ, int NT, bool FUSED>
 __global__ void __launch_bounds__(NT, 2) k_fft_pass_d(const cpx<double>* __restrict__ in,
                                                       cpx<double>* __restrict__ out, PassArgs a,
@@ -1019,6 +1019,8 @@ FC2_D void regpass_body(const cpx<float>* __restrict__ in, cpx<float>* __restric
     constexpr int R = 1 << LOGR, J = 1 << LOGJ, E = R * J, NT = RB == 64 ? P64_NT : P32_NT;
     constexpr int QAB = LOGR - LRB, QA = 1 << QAB;
     constexpr int PERA = RB / QA;  // stage-A butterflies per thread
+    // (the first 2^10 pass of the radix-64 family is k_fft_first10)
+    const bool first = !(RB == 64 && LOGR == 10) && a.first;
     static_assert(RB == 64 || RB == 32, "stage-B radix 64 or 32");
     static_assert(E == RB * NT, "tile must be RB elements per thread");
     static_assert(PERA * NT == RB * J, "stage-A butterflies must divide evenly");
@@ -1035,7 +1037,7 @@ FC2_D void regpass_body(const cpx<float>* __restrict__ in, cpx<float>* __restric
     cp_async_wait_all();
     auto rows_of = [&](int g) {
         int rows = R;
-        if (a.first) {
+        if (first) {
             const int L = (int)Lg[g];
             rows = (L + S - 1) / S;
             if (rows > R) rows = R;
@@ -1054,7 +1056,7 @@ FC2_D void regpass_body(const cpx<float>* __restrict__ in, cpx<float>* __restric
             if (tn < ntiles) {
                 const int gnl = tn / tiles_x, bn = tn - gnl * tiles_x, gn = a.g0 + gnl;
                 const cpx<T>* ginn = in + (int64_t)gn * M;
-                if (!a.first) {
+                if (!first) {
                     constexpr int CH = 4096;  // bytes per prefetch request
                     constexpr int NCH = E * (int)sizeof(cpx<T>) / CH;
                     const char* base = reinterpret_cast<const char*>(ginn + (int64_t)bn * E);
@@ -1085,7 +1087,7 @@ FC2_D void regpass_body(const cpx<float>* __restrict__ in, cpx<float>* __restric
                     }
                     PrunedDFT<T, QA, MZ>::run(v);
                 } else {
-                    if (a.first) {
+                    if (first) {
 #pragma unroll
                         for (int k = 0; k < QA; ++k) {
                             const int r = pp + k * RB;
@@ -1126,7 +1128,7 @@ FC2_D void regpass_body(const cpx<float>* __restrict__ in, cpx<float>* __restric
             }
         };
         int mz = QA;
-        if (a.first) {
+        if (first) {
             const int kz = (rows + RB - 1) >> LRB;
             mz = 1;
             while (mz < kz && mz < QA) mz <<= 1;
@@ -1545,7 +1547,7 @@ __global__ void __launch_bounds__(PT_NT, 1) k_fft_pass_tma(const cpx<float>* __r
 
 // ------------------------------------------- the 2^8 and 2^9 bulk-copy passes
 // The passes of radix 2^8 and 2^9 with the stages and arithmetic of
-// k_fft_pass_tma (16 x 16 and 32 x 16; results are bit-equal), by two groups of
+// k_fft_pass_tma (16 x 16 and 32 x 16), by two groups of
 // 256 threads per SM, each on a tile of its own.  A transform of one tile is a
 // chain -- wait for its copy, stage 1, barrier, last stage, store -- and with
 // one tile per SM in lockstep each link idles what the others need (issue
@@ -1842,7 +1844,7 @@ __global__ void __launch_bounds__(DUO_NT, 1) k_fft_pass_duo(const cpx<float>* __
 
 // ------------------------------------------- the 2^10 first pass
 // The first pass of radix 2^10 with the arithmetic of k_fft_pass64 (stage A
-// radix 16, stage B radix 64; results are bit-equal), by three groups of 128
+// radix 16, stage B radix 64), by three groups of 128
 // threads per SM with an 8-column tile each: a thread holds 64 elements in 167
 // registers, and one group's loads, barriers and stores are covered by the other
 // two's arithmetic, where one group of 256 threads with one 16-column tile
