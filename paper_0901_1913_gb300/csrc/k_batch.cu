@@ -201,18 +201,24 @@ constexpr double BX_EPS_DF = 1.5e-12;  // relative precision of the tier-2 (doub
 // nearly singular and starts at the double tier
 constexpr double BX_DMIN_T3 = 1e-7;
 // Smallest relative pivot used for routing.  Curves of fewer than 8 harmonics
-// count as nearly singular whatever their pivots (the empty columns of a system
-// padded to 8 do), so their flagged entries go straight to the last and most
-// precise tier, whichever capacity the solve is padded to.
+// count as nearly singular whatever their pivots, so their flagged entries all go
+// to the last and most precise tier, whichever capacity the solve is padded to.
+// (The pivots of a padded system would make the route depend on its padding: the
+// empty harmonics' columns have diagonal 1/2 and couple to the curve's own, so in
+// nearly singular equations theirs mostly come out negative, but not always -- in
+// 1024 survey curves routed by the smallest pivot of the system padded to 8, 17 of
+// some 30000 entries went to the float and double-float tiers.)
 FC2_D double bx_pivot(double dmin, int H) { return H < 8 ? 0.0 : dmin; }
 
 // Double re-solve of listed (curve, bin) entries of the float path.  Entries
 // still too sensitive go on to the exact sums: to the float tier, straight to
 // the double-float tier when the float sums could not settle them either
 // (error estimate at the float sums' precision above the bar, or a small
-// relative pivot), or straight to the double tier when the coefficient norm
+// relative pivot), or straight to the last tier when the coefficient norm
 // is beyond the double-float sums as well or the pivot is below what the
-// gridded equations resolve.
+// gridded equations resolve.  bx_pivot sends those of curves of fewer than 8
+// harmonics to the last tier: the float and double-float tiers serve the mixed
+// path's curves of 8 harmonics, and FP64 entries on their way to the double tier.
 template <int HM>
 __global__ void __launch_bounds__(128) k_bresolve(const cpx<float>* __restrict__ spec,
                                                   const float* __restrict__ dec, int64_t N,
