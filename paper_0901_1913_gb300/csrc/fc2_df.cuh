@@ -337,8 +337,9 @@ FC2_D void fx_flush(long long& acc, float h, float l, float scale) {
 // group stages its samples' phases u_i = A_i + ju B_i (mod 2^64) and weights in
 // shared memory one tile (qt of a block's samples for both halves) ahead, and
 // the next sample's table values are fetched a step ahead.  Bound by the float
-// pipe (two thirds busy; about 100 warp instructions per sample and multiple,
-// half of them packed) together with the load unit (the scattered table reads).
+// pipe (59% active; about 100 warp instructions per sample and multiple, half of
+// them packed) together with L1 (74%: the scattered reads of the large table);
+// the one-warp form, on shared-memory tables, 46% and 25% in a short launch.
 // One lane per multiple with every load, phase and 64-bit conversion of its own
 // took 177 instructions and waited on its loads:
 //   plan of n = 10^6, H = 8, N = 2^25 (481 bins): 66.3 -> 34.2 ms

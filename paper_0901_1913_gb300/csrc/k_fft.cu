@@ -656,7 +656,8 @@ FC2_HD constexpr int stage_tw_offset(int LOGR, int DONE) {
 
 // ------------------------------------------------------- double-precision pass
 // Bound by the double pipe (a warp's double instruction takes 64 clocks of its
-// sub-partition), so what counts is the double operations per element:
+// sub-partition; 92 and 93% active in the 2^10 and 2^9 passes of eight survey
+// curves), so what counts is the double operations per element:
 //   * every level of every stage is a radix-2 butterfly a +- w b of six fused
 //     operations (three per element and bit), with all of the element's
 //     twiddles in w: a stage of radix Q after passes of radix product D and
@@ -1547,8 +1548,8 @@ __global__ void __launch_bounds__(PT_NT, 1) k_fft_pass_tma(const cpx<float>* __r
 
 // ------------------------------------------- the 2^8 and 2^9 bulk-copy passes
 // The passes of radix 2^8 and 2^9 with the stages and arithmetic of
-// k_fft_pass_tma (16 x 16 and 32 x 16), by two groups of
-// 256 threads per SM, each on a tile of its own.  A transform of one tile is a
+// k_fft_pass_tma (16 x 16 and 32 x 16), by two groups of 256 threads per SM, each
+// on a tile of its own.  A transform of one tile is a
 // chain -- wait for its copy, stage 1, barrier, last stage, store -- and with
 // one tile per SM in lockstep each link idles what the others need (issue
 // active 54%, and the 32 x 16 pass's 256 first butterflies left half of 512
@@ -1562,7 +1563,8 @@ __global__ void __launch_bounds__(PT_NT, 1) k_fft_pass_tma(const cpx<float>* __r
 // leave in runs of the next pass's layout.  A first pass skips the butterfly
 // levels whose second operands are zero padding; a middle pass before the last
 // one stores straight from registers, contiguous along the columns.
-// Bound by memory: the later passes run at 6.0-6.1 TB/s, 0.88 of the copy rate.
+// Bound by memory: the later passes run at 6.0-6.1 TB/s, 0.88 of the copy rate (24
+// survey curves under ncu: 5.6 TB/s, issue 50% and float pipe 48% active).
 //   1024 survey curves, second pass 2^9:  17.7 -> 12.95 ms
 //   24 grids of 2^26: both 2^9 passes 18.0 -> 3.6 + 4.2 ms (the middle one 10.7
 //     with its results staged), last 2^8 4.2 -> 3.2 ms
@@ -1844,12 +1846,13 @@ __global__ void __launch_bounds__(DUO_NT, 1) k_fft_pass_duo(const cpx<float>* __
 
 // ------------------------------------------- the 2^10 first pass
 // The first pass of radix 2^10 with the arithmetic of k_fft_pass64 (stage A
-// radix 16, stage B radix 64), by three groups of 128
-// threads per SM with an 8-column tile each: a thread holds 64 elements in 167
-// registers, and one group's loads, barriers and stores are covered by the other
-// two's arithmetic, where one group of 256 threads with one 16-column tile
-// waited for itself (issue active 47%).  Bound by the shared-memory and issue
-// rates together (without its stores it takes 9% less, without its loads 18%).
+// radix 16, stage B radix 64), by three groups of 128 threads per SM with an
+// 8-column tile each: a thread holds 64 elements in 164 registers, and one
+// group's loads, barriers and stores are covered by the other two's arithmetic,
+// where one group of 256 threads with one 16-column tile waited for itself.
+// Bound by latency with 12 warps an SM: 24 survey curves (1.4 GB) take 0.33 ms
+// under ncu, 0.62 of the copy rate, with issue 39% and the float pipe 35% active,
+// the warps waiting for the store queue, their loads and shared memory alike.
 // The tile has one slot of padding per two rows (16 columns of 8 bytes: all
 // banks): the column-wise and the row-wise accesses are free of conflicts, and
 // every access of an unrolled loop is a fixed offset from its thread's base.
