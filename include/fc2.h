@@ -231,6 +231,10 @@ fc2_status fc2_execute(fc2_plan p, double* dchi2, fc2_best* best, fc2_best* peak
  *     sum_{c' < c} H_c' N_c'.  Host or device per outputs_on_device.  May be NULL.
  *   peaks [C][top_k] (host): per-curve peak records as fc2_execute.  May be NULL.
  * Validation as fc2_plan_create for each curve.
+ * With FC2_PREC_FP64 the normal equations are scaled by factors held in float
+ * (6e-8): at nearly singular bins (periods longer than the span) Delta chi^2 may
+ * be off by some hundredths of chi2_0, where a plan of fc2_plan_create or the
+ * mixed path, which recompute those bins, are not.
  */
 fc2_status fc2_execute_batched(int64_t C, const int64_t* offsets,
                                const double* t, const double* x, const double* sigma,

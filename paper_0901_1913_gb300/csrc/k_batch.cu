@@ -38,6 +38,9 @@ struct CurveTab {
     const double* scal;     // [C][SC_COUNT]
     const int* slot0;       // [C] first transform slot of the curve
     const int64_t* out_off; // [C] first output element of the curve
+    // (FP64 batches too: Q_0 = 1 beside sums scaled by a rounded 1/W leaves 6e-8 in
+    // their systems, which the error estimate does not know; nearly singular bins
+    // are not recomputed and show it)
     const float* sq;        // [C] 1/W
     const float* sp;        // [C] 1/sqrt(W chi2_0)
     const float* s1n;       // [C] sum w(x - xbar) / sqrt(W chi2_0)

@@ -1563,8 +1563,8 @@ __global__ void __launch_bounds__(PT_NT, 1) k_fft_pass_tma(const cpx<float>* __r
 // leave in runs of the next pass's layout.  A first pass skips the butterfly
 // levels whose second operands are zero padding; a middle pass before the last
 // one stores straight from registers, contiguous along the columns.
-// Bound by memory: the later passes run at 6.0-6.1 TB/s, 0.88 of the copy rate (24
-// survey curves under ncu: 5.6 TB/s, issue 50% and float pipe 48% active).
+// Bound by memory: the survey's second pass runs at 6.3 TB/s, 0.92 of the copy rate
+// (in a short launch, 24 curves: 5.6 TB/s, issue 50% and float pipe 48% active).
 //   1024 survey curves, second pass 2^9:  17.7 -> 12.95 ms
 //   24 grids of 2^26: both 2^9 passes 18.0 -> 3.6 + 4.2 ms (the middle one 10.7
 //     with its results staged), last 2^8 4.2 -> 3.2 ms
@@ -1850,9 +1850,10 @@ __global__ void __launch_bounds__(DUO_NT, 1) k_fft_pass_duo(const cpx<float>* __
 // 8-column tile each: a thread holds 64 elements in 164 registers, and one
 // group's loads, barriers and stores are covered by the other two's arithmetic,
 // where one group of 256 threads with one 16-column tile waited for itself.
-// Bound by latency with 12 warps an SM: 24 survey curves (1.4 GB) take 0.33 ms
-// under ncu, 0.62 of the copy rate, with issue 39% and the float pipe 35% active,
-// the warps waiting for the store queue, their loads and shared memory alike.
+// Bound by latency with 12 warps an SM: the survey's first pass runs at 4.7 TB/s,
+// 0.69 of the copy rate; in a short launch (24 curves, 4.2 TB/s) issue is 39% and
+// the float pipe 35% active, the warps waiting for the store queue, their loads
+// and shared memory alike.
 // The tile has one slot of padding per two rows (16 columns of 8 bytes: all
 // banks): the column-wise and the row-wise accesses are free of conflicts, and
 // every access of an unrolled loop is a fixed offset from its thread's base.
