@@ -460,10 +460,13 @@ FC2_HD bool one_stride(const PassArgs& a, int LOGR, int LOGJ, int NT) {
 FC2_HD bool middle_direct(const PassArgs& a, int LOGR, int LOGJ) {
     return !a.last && a.logNs + LOGR + a.logRn == a.logM && a.logNs >= a.logJn && a.logNs >= LOGJ;
 }
-// k_fft_first10 before a last pass of 16-column tiles: the 16 rows of a half-warp
-// are one 128-byte line of its layout (24 grids of 2^20: both passes 264 us with
-// the results staged, 249 so; 207 and 198 with one row in a thousand occupied).
-FC2_HD bool first10_direct(const PassArgs& a) { return two_pass(a, 10) && a.logJn == 4; }
+// k_fft_first10 before a last pass of 16-column tiles (radix 2^9 and 2^10): the 16
+// rows of a half-warp are one 128-byte line of its layout (24 grids of 2^20: both
+// passes 263 us with the results staged, 239 so; 206 and 186 with one row in a
+// thousand occupied).
+FC2_HD bool first10_direct(const PassArgs& a) {
+    return two_pass(a, 10) && a.logJn == 4 && (a.logRn == 9 || a.logRn == 10);
+}
 
 // Last pass: mode m of grid g goes to its place in the spectra.  Grid
 // g < npk (packed) stores F(sh + j) at [2g][j] and F(-(sh + j)) at [2g + 1][j];
@@ -1942,10 +1945,15 @@ __global__ void __launch_bounds__(D10_NG * D10_GT, 1) k_fft_first10(const cpx<fl
         for (int k = 1; k < 64; ++k) v[k] = mul(v[k], st[(k - 1) * QA + pp]);
         SmallDFT<T, 64>::run(v);
         if (direct) {  // rows 16 k + pp: block k, row pp of it
-            cpx<T>* dst = gout + ((int64_t)(j0 + jj) << 4) + pp;
-            const int64_t blk = 1ll << (a.logRn + 4);
+            // (the block's length as a constant puts the offsets into the store
+            // instructions: computed, 249 us instead of 239 for 24 grids of 2^20)
+            cpx<T>* dst = gout + ((j0 + jj) << 4) + pp;
+            auto store = [&](auto blk) {
 #pragma unroll
-            for (int k = 0; k < 64; ++k) dst[k * blk] = v[k];
+                for (int k = 0; k < 64; ++k) dst[k << decltype(blk)::value] = v[k];
+            };
+            if (a.logRn == 9) store(std::integral_constant<int, 13>{});
+            else store(std::integral_constant<int, 14>{});
         } else {
             d10_sync(grp);
 #pragma unroll
